@@ -309,17 +309,34 @@ __global__ void k_adam(long n, float* w, const float* g, float* m, float* v, flo
     w[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
-// BF16 copies: wb[t][co_pad][ci_pad] = W[t][co][ci]; wt[t][ci_pad][co_pad] = W[T-1-t][co][ci]
+// output channels of one CTA of the tcgen05 convolution with n output channels
+__host__ __device__ constexpr int conv_nb(int n) {
+    return n % 64 == 0 ? 64 : n % 48 == 0 ? 48 : n % 32 == 0 ? 32 : 16;
+}
+// element of tap t, output channel o (of n), input channel i (of cin) in the tcgen05 convolution's weights:
+// [block of NB][block of 16 input channels][tap (dy, dx)][dz = +1, 0, -1][8 channels][2 x 8 inputs][8][8]
+__device__ __forceinline__ size_t conv_w_at(int t, int o, int n, int i, int cin) {
+    const int NB = conv_nb(n), row = (2 - t / 9) * NB + o % NB;
+    const size_t blk = (size_t)(o / NB) * (cin / 16) + i / 16;
+    return (blk * 9 + t % 9) * (3 * NB * 16) + (row >> 3) * 128 + ((i >> 3) & 1) * 64 + (row & 7) * 8 + (i & 7);
+}
+
+// BF16 copies: wb[t][co_pad][ci_pad] = W[t][co][ci]; wt[t][ci_pad][co_pad] = W[T-1-t][co][ci]; for 27 taps
+// also both in the order of the tcgen05 convolution (wk, wkt)
 __global__ void k_weights_bf16(const float* W, int taps, int cout, int cin, int co_pad, int ci_pad, bf16* wb,
-                               bf16* wt) {
+                               bf16* wt, bf16* wk, bf16* wkt) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long n = (long)taps * co_pad * ci_pad;
     if (i >= n) return;
     const int ci = (int)(i % ci_pad), co = (int)((i / ci_pad) % co_pad), t = (int)(i / ((long)ci_pad * co_pad));
-    const float val = (co < cout && ci < cin) ? W[((size_t)t * cout + co) * cin + ci] : 0.f;
-    wb[i] = __float2bfloat16(val);
+    const bf16 val = __float2bfloat16((co < cout && ci < cin) ? W[((size_t)t * cout + co) * cin + ci] : 0.f);
+    wb[i] = val;
     const int tf = taps - 1 - t;
-    wt[((size_t)tf * ci_pad + ci) * co_pad + co] = __float2bfloat16(val);
+    wt[((size_t)tf * ci_pad + ci) * co_pad + co] = val;
+    if (taps == 27) {
+        wk[conv_w_at(t, co, co_pad, ci, ci_pad)] = val;
+        wkt[conv_w_at(tf, ci, ci_pad, co, co_pad)] = val;
+    }
 }
 
 __global__ void k_input_host(int N, const double* x2, bf16* x) {  // x2: [N][2] from the host
@@ -377,32 +394,45 @@ unsigned blocks(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 // ---------------------------------------------------------------------------
 // 3x3x3 convolution on the 5th-generation tensor cores (tcgen05).
 //
-// One CTA of 128 threads computes output tiles of 8 (x) x 16 (y) x 2 (z)
-// voxels for all N output channels: two M = 128 GEMMs (one per z plane) whose
-// FP32 accumulators D[128][N] live side by side in tensor memory (TMEM lane m
-// = voxel m of the plane, column zp N + n = channel n).  The work of a tile is
-// a sequence of steps (16-input-channel block cb, nine taps t0 .. t0+8).  For
-// each channel block the CTA stages the input tile with a one-voxel halo
-// (10 x 18 x 4 voxels) in shared memory once, and every tap of both planes
-// reads its A operand from it: tap (dz, dy, dx) is the tile shifted by whole
-// 16-byte rows, so it only changes the start address of the shared-memory
-// matrix descriptor.  Halo tiles and weight blocks are double-buffered and
-// filled with cp.async while the tensor core works on the previous step; one
-// thread issues the MMAs (tcgen05.mma.cta_group::1.kind::f16: BF16 A and B,
-// FP32 D, M = 128, K = 16) and commits them to the step's mbarrier, and a
-// buffer is refilled only after the MMAs that read it have completed.
-// Operands use the canonical K-major layout without swizzling: a core matrix
-// is 8 rows of 16 bytes (8 channels) stored contiguously; the descriptor's
-// leading offset steps to the next 8 channels, its stride offset to the next
-// 8 rows.
+// What bounds it: an M = 128, K = 16 BF16 MMA reads 4 KB of A and 32 N bytes
+// of B from shared memory at 128 B a cycle and multiplies for N / 2 cycles, so
+// with N = 16 (the layers of the finest level) it is bound by the A reads
+// (36 cycles for 8 of arithmetic).  The kernel therefore folds the three dz
+// taps into N: an input plane meets the weights of all three in one MMA of
+// N = 3 NB columns, whose column blocks are the accumulators of the output
+// planes below, at and above it, which lie side by side in tensor memory.
+//
+// A CTA (one per SM, persistent) computes tiles of 8 (x) x 16 (y) x zt voxels
+// for a block of NB output channels: accumulator column j NB + c of tensor
+// memory lane m is channel c of voxel m of output plane j.  Its work is a
+// sequence of stages, one a 16-input-channel block: the input tile with a
+// one-voxel halo (zt + 2 planes of 18 x 10 voxels) and the block's weights of
+// all 27 taps, both in the canonical K-major layout without swizzling (a core
+// matrix is 8 rows of 16 bytes stored contiguously; the descriptor's leading
+// offset steps to the next 8 channels, its stride offset to the next 8 rows).
+// A tap (dy, dx) only shifts the start address of the A descriptor by whole
+// 16-byte rows.  Input plane zi feeds output planes zi-2 .. zi of the tile
+// (clipped at its ends), a contiguous window of the column blocks and of the
+// weight rows, stored in the order dz = +1, 0, -1.  Every accumulator still
+// receives its products in the order channel block, dz, dy, dx.
+//
+// Roles: warps 0-3 read the accumulators of a finished tile (bias, ReLU, BF16
+// rounding, 16-byte stores), warp 4 issues the MMAs (one thread), warps 5-7
+// stage the input with cp.async, one thread of them the weights with one bulk
+// copy a stage.  Stages form a ring of 2 to 4 buffers, accumulators two sets,
+// so copies, MMAs and read-out of consecutive tiles overlap.  zt is chosen by
+// conv_planes (below).
+//
+// Measured, forward pass of the network (GB300): 256^3 8.05 -> 3.50 ms, 128^3
+// 1.20 -> 0.52 ms, 40 x 24 x 16 283 -> 107 us against one MMA of N = NB a tap
+// and plane with a CTA barrier every 18 MMAs; bit-identical.
 // ---------------------------------------------------------------------------
-constexpr int kTcThreads = 128;
-constexpr int kTileX = 8, kTileY = 16, kTileZ = 2;
-constexpr int kHX = kTileX + 2, kHY = kTileY + 2, kHZ = kTileZ + 2, kKC = 2;  // halo; 16 channels = 2 x 8
-constexpr int kHaloUnits = kHZ * kHY * kKC * kHX;                            // 16-byte units
-constexpr int kHaloBytes = kHaloUnits * 16;
-constexpr int kGuardBytes = 4096;
-constexpr int kTapsPerIter = 9;
+constexpr int kZbThreads = 256, kZbProd = 96, kZbMmaWarp = 4;
+constexpr int kTileX = 8, kTileY = 16;
+constexpr int kHX = kTileX + 2, kHY = kTileY + 2;
+constexpr int kPlaneUnits = kHY * 2 * kHX;       // 16-byte units of one staged plane: [y][8-channel half][x]
+constexpr int kPlaneBytes = kPlaneUnits * 16;
+constexpr int kZbMaxStages = 4;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -492,38 +522,92 @@ __device__ __forceinline__ void cp_async16(uint32_t saddr, const void* g, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// tcgen05 convolution: out[v][co] = act(bias[co] + sum_t sum_ci in[v + off(t)][ci] w[t][co][ci]) for
-// co < cout (BF16 out, row stride out_stride); cin and N multiples of 16, N <= 256; ncols: TMEM
-// columns (a power of two >= max(32, 2N)).  With up != NULL the input is the concatenation
-// [nearest upsampling of up (cup channels, on the grid of half the extents), in (cin - cup channels)],
-// gathered while staging instead of being stored.  On a wait that runs out, *err is set to 1 and
-// the CTA stops.  Tensor memory is released only once every MMA the CTA committed has been seen
-// complete: a barrier whose wait gave up is waited for again (poll-bounded) before the dealloc;
-// if an MMA is still unconfirmed then, *err is set to 2 (the CTA must still release its columns
-// before it exits, so their contents are not to be trusted by any later kernel of the context).
-__global__ void __launch_bounds__(kTcThreads) k_conv_tc(CG g, const bf16* __restrict__ in, int cin,
-                                                        const bf16* __restrict__ up, int cup,
-                                                        const bf16* __restrict__ w, int N,
-                                                        const float* __restrict__ bias, int cout, bf16* out,
-                                                        int out_stride, int relu, int ncols, int* err) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
-    const int bunits = kTapsPerIter * 2 * N;  // 16-byte units of one weight buffer
-    const uint32_t halo_addr = smem_u32(smem);                                   // 2 halo buffers
-    const uint32_t b_addr = smem_u32(smem + 2 * kHaloBytes + kGuardBytes);       // 2 weight buffers
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// 16 consecutive FP32 columns of this thread's TMEM lane (no wait)
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
+                 "r"(bytes)
+                 : "memory");
+}
+// bulk copy of bytes (a multiple of 16) from 16-byte aligned global memory, counted on bar
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+// mbar_wait_bounded that also ends (false) once another role of the CTA has given up
+__device__ __forceinline__ bool mbar_wait_role(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+    const unsigned long long t0 = tc_globaltimer();
+    long polls = 0;
+    while (!mbar_try_wait(bar, parity)) {
+        if (*abort_flag) return false;
+        if (++polls > (1L << 20) && tc_globaltimer() - t0 > 1000000000ull) {
+            *abort_flag = 1;
+            atomicMax(err, 1);
+            return false;
+        }
+    }
+    return true;
+}
 
-    if (warp == 0) {
+struct ConvArgs {
+    CG g;
+    const bf16* in;     // [voxel][cin - cup]
+    const bf16* up;     // coarse input of the first cup channels (nearest upsampling of half the extents), or null
+    int cin, cup;       // multiples of 16
+    const bf16* w;      // blocked weights (k_weights_bf16): [channel block of NB][16 input channels][9][3 NB][16]
+    const float* bias;  // [N] or null
+    bf16* out;          // [voxel][N]
+    int N, relu;
+    int zt, nstage, nblk, ncols;  // planes of a tile, staging buffers, N / NB, TMEM columns (a power of two >= 2 zt NB)
+    int* err;
+};
+
+// out[v][co] = act(bias[co] + sum_t sum_ci in[v + off(t)][ci] w[t][co][ci]).  A wait that runs out sets
+// *err to 1, and every role of the CTA stops.  Tensor memory is released only once every MMA the CTA
+// issued has been seen complete (a last commit, waited for with a poll bound); if that wait runs out too,
+// *err is set to 2 (the CTA must still release its columns before it exits, so their contents are not to
+// be trusted by any later kernel of the context).
+template <int NB>
+__global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t b_full[kZbMaxStages], b_wfull[kZbMaxStages], b_empty[kZbMaxStages];
+    __shared__ __align__(8) uint64_t b_acc[2], b_accfree[2], b_end;
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_abort;
+    const CG& g = a.g;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t kWBytes = 27u * 32u * NB;
+    const uint32_t stage_bytes = kWBytes + (uint32_t)((a.zt + 2) * kPlaneBytes);
+    const uint32_t base = smem_u32(smem);
+
+    if (warp == kZbMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(ncols)
+                     "r"(a.ncols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
+        for (int i = 0; i < kZbMaxStages; ++i) {
+            mbar_init(&b_full[i], kZbProd);
+            mbar_init(&b_wfull[i], 1);
+            mbar_init(&b_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&b_acc[i], 1);
+            mbar_init(&b_accfree[i], 128);
+        }
+        mbar_init(&b_end, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -531,151 +615,177 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(CG g, const bf16* __rest
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t idesc = idesc_bf16(128, N);
 
     const int tiles_x = (g.nx + kTileX - 1) / kTileX, tiles_y = (g.ny + kTileY - 1) / kTileY;
-    const int tiles_z = (g.nz + kTileZ - 1) / kTileZ;
-    const long ntiles = (long)tiles_x * tiles_y * tiles_z;
-    const int ncb = cin / 16, steps_per_cb = 27 / kTapsPerIter;
-    const int steps_per_tile = ncb * steps_per_cb;
-    // this CTA's tiles: blockIdx.x, blockIdx.x + gridDim.x, ...; its steps are numbered 0, 1, ...
-    const long my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const long nsteps = my_tiles * steps_per_tile;
-    uint32_t phase[2] = {0u, 0u};
-    bool pending[2] = {false, false};
-    bool unconfirmed[2] = {false, false};   // a wait on this barrier gave up (phase uphase[b])
-    uint32_t uphase[2] = {0u, 0u};
+    const int tiles_z = (g.nz + a.zt - 1) / a.zt;
+    const int items = tiles_x * tiles_y * tiles_z * a.nblk;  // item = tile nblk + channel block
+    const int ncb = a.cin / 16;
+    auto origin = [&](int item, int& x0, int& y0, int& z0, int& blk) {
+        const int tile = item / a.nblk;
+        blk = item - tile * a.nblk;
+        const int r = tile / tiles_x;
+        x0 = (tile - r * tiles_x) * kTileX;
+        const int tz = r / tiles_y;
+        y0 = (r - tz * tiles_y) * kTileY;
+        z0 = tz * a.zt;
+    };
 
-    auto tile_origin = [&](long k, int& x0, int& y0, int& z0) {
-        const long tile = blockIdx.x + k * gridDim.x;
-        const long tz = tile / ((long)tiles_x * tiles_y);
-        const int rem = (int)(tile - tz * tiles_x * tiles_y);
-        z0 = (int)tz * kTileZ;
-        y0 = (rem / tiles_x) * kTileY;
-        x0 = (rem % tiles_x) * kTileX;
-    };
-    // wait for the MMAs committed to mbarrier b (every thread; a wait that runs out sets s_abort)
-    auto wait_mma = [&](int b) {
-        if (pending[b]) {
-            if (!mbar_wait_bounded(&mbar[b], phase[b])) {
-                s_abort = 1;
-                atomicExch(err, 1);
-                unconfirmed[b] = true;
-                uphase[b] = phase[b];
-            }
-            phase[b] ^= 1u;
-            pending[b] = false;
-        }
-    };
-    // issue the cp.async loads of step s: the halo tile when s starts a channel block, and the weights
-    auto load_step = [&](long s) {
-        const long k = s / steps_per_tile;
-        const int r = (int)(s - k * steps_per_tile), cbi = r / steps_per_cb, t0 = (r % steps_per_cb) * kTapsPerIter;
-        const int cb = cbi * 16;
-        if (t0 == 0) {
-            int x0, y0, z0;
-            tile_origin(k, x0, y0, z0);
-            const uint32_t hbase = halo_addr + (uint32_t)(((k * ncb + cbi) & 1) * kHaloBytes);
-            for (int u = tid; u < kHaloUnits; u += kTcThreads) {
-                const int hx = u % kHX, r1 = u / kHX, kc = r1 % kKC, r2 = r1 / kKC, hy = r2 % kHY, hz = r2 / kHY;
-                const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z0 + hz - 1;
-                const bool ok = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny && gz >= 0 && gz < g.nz;
-                const int c = cb + kc * 8;
-                const bf16* src = in;
-                if (ok) {
-                    if (c < cup)
-                        src = up + ((size_t)((long)(gz >> 1) * (g.ny >> 1) + (gy >> 1)) * (g.nx >> 1) + (gx >> 1)) * cup +
-                              c;
-                    else
-                        src = in + ((size_t)((long)gz * g.ny + gy) * g.nx + gx) * (cin - cup) + (c - cup);
+    if (warp > kZbMmaWarp) {
+        // ---- staging ----
+        const int pt = tid - (kZbMmaWarp + 1) * 32;
+        int st = 0, issued = 0;
+        uint32_t ph = 1u;  // a buffer's first use finds it empty
+        bool ok = true;
+        uint64_t* prev = nullptr;
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+            int x0, y0, z0, blk;
+            origin(item, x0, y0, z0, blk);
+            for (int cb = 0; cb < ncb; ++cb) {
+                ok = mbar_wait_role(&b_empty[st], ph, &s_abort, a.err);
+                if (!ok) break;
+                const uint32_t wbase = base + (uint32_t)st * stage_bytes, hbase = wbase + kWBytes;
+                if (pt == 0) {
+                    mbar_arrive_tx(&b_wfull[st], kWBytes);
+                    bulk_load(wbase, a.w + (size_t)(blk * ncb + cb) * (kWBytes / 2), kWBytes, &b_wfull[st]);
+                    ++issued;
                 }
-                cp_async16(hbase + (uint32_t)u * 16u, src, ok);
+                const bool isup = cb * 16 < a.cup;
+                const int sh = isup ? 1 : 0, C = isup ? a.cup : a.cin - a.cup;
+                const int snx = g.nx >> sh, sny = g.ny >> sh;
+                const bf16* src0 = (isup ? a.up + cb * 16 : a.in + (cb * 16 - a.cup));
+                const size_t zstride = (size_t)snx * sny * C;
+                for (int u = pt; u < kPlaneUnits; u += kZbProd) {
+                    const int kc = u & 1, r = u >> 1, hy = r / kHX, hx = r - hy * kHX;
+                    const int gx = x0 + hx - 1, gy = y0 + hy - 1;
+                    const bool in2 = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny;
+                    const bf16* p = src0 + (in2 ? ((size_t)(gy >> sh) * snx + (gx >> sh)) * C : 0) + kc * 8;
+                    uint32_t dst = hbase + (uint32_t)((hy * 2 + kc) * kHX + hx) * 16u;
+                    for (int hz = 0; hz < a.zt + 2; ++hz, dst += kPlaneBytes) {
+                        const int gz = z0 + hz - 1;
+                        const bool in3 = in2 && gz >= 0 && gz < g.nz;
+                        cp_async16(dst, in3 ? p + (size_t)(gz >> sh) * zstride : a.in, in3);
+                    }
+                }
+                cp_async_commit();
+                // hand over the stage before this one: its copies are done when at most one group is open
+                if (prev) {
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    fence_proxy_async();
+                    mbar_arrive(prev);
+                }
+                prev = &b_full[st];
+                if (++st == a.nstage) {
+                    st = 0;
+                    ph ^= 1u;
+                }
             }
         }
-        const uint32_t bbase = b_addr + (uint32_t)((s & 1) * bunits * 16);
-        for (int u = tid; u < bunits; u += kTcThreads) {
-            const int t = u / (2 * N), rr = u - t * 2 * N;
-            const int ng = rr >> 4, kc = (rr >> 3) & 1, n = ng * 8 + (rr & 7);
-            cp_async16(bbase + (uint32_t)u * 16u, w + ((size_t)(t0 + t) * N + n) * cin + cb + kc * 8, true);
-        }
-        cp_async_commit();
-    };
-
-    if (nsteps > 0) load_step(0);
-    for (long s = 0; s < nsteps; ++s) {
-        const long k = s / steps_per_tile;
-        const int r = (int)(s - k * steps_per_tile), cbi = r / steps_per_cb, t0 = (r % steps_per_cb) * kTapsPerIter;
-        // operands of step s are in shared memory
         cp_async_wait_all();
-        fence_proxy_async();
-        __syncthreads();
-        if (s_abort) break;
-        if (tid == 0) {
-            tc_fence_after();
-            const uint32_t hbase = halo_addr + (uint32_t)(((k * ncb + cbi) & 1) * kHaloBytes);
-            const uint32_t bbase = b_addr + (uint32_t)((s & 1) * bunits * 16);
-#pragma unroll 1
-            for (int t = 0; t < kTapsPerIter; ++t) {
-                const int tap = t0 + t;
-                const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                const uint64_t bd = smem_desc(bbase + (uint32_t)(t * 2 * N) * 16u, 8 * 16, kKC * 8 * 16);
-#pragma unroll
-                for (int zp = 0; zp < kTileZ; ++zp) {
-                    const int u0 = ((zp + 1 + dz) * kHY + (1 + dy)) * kKC * kHX + (1 + dx);
-                    const uint64_t ad = smem_desc(hbase + (uint32_t)u0 * 16u, kHX * 16, kKC * kHX * 16);
-                    tc_mma(tmem + (uint32_t)(zp * N), ad, bd, idesc, (r == 0 && t == 0) ? 0u : 1u);
-                }
-            }
-            tc_commit(&mbar[s & 1]);
+        if (prev) {
+            fence_proxy_async();
+            mbar_arrive(prev);
         }
-        pending[s & 1] = true;
-        // the buffers of step s+1 were last read by step s-1: wait for it, then prefetch step s+1
-        wait_mma((int)((s + 1) & 1));
-        if (s + 1 < nsteps) load_step(s + 1);
-        if (r == steps_per_tile - 1) {
-            // last step of the tile: accumulators complete once step s's MMAs are
-            wait_mma((int)(s & 1));
-            __syncthreads();
-            if (s_abort) break;
-            tc_fence_after();
-            int x0, y0, z0;
-            tile_origin(k, x0, y0, z0);
-            const int m = warp * 32 + lane;
-            const int gx = x0 + (m & 7), gy = y0 + (m >> 3);
-            for (int zp = 0; zp < kTileZ; ++zp) {
-                const int gz = z0 + zp;
-                const bool inside = gx < g.nx && gy < g.ny && gz < g.nz;
-                bf16* orow =
-                    out + ((size_t)((long)(inside ? gz : 0) * g.ny + (inside ? gy : 0)) * g.nx + (inside ? gx : 0)) *
-                              out_stride;
-                for (int c0 = 0; c0 < N; c0 += 8) {
-                    float v[8];
-                    tmem_ld8(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(zp * N + c0), v);
-                    if (inside && c0 + 8 <= cout) {
-                        __align__(16) bf16 o[8];
+        // after an abort the bulk copies in flight are waited for (bounded) before the CTA may end
+        if (pt == 0 && s_abort)
+            for (int i = max(0, issued - a.nstage); i < issued; ++i)
+                mbar_drain(&b_wfull[i % a.nstage], (uint32_t)(i / a.nstage) & 1u);
+    } else if (warp == kZbMmaWarp) {
+        // ---- MMA issue ----
+        if (lane == 0) {
+            int st = 0, k = 0;
+            uint32_t ph = 0u;
+            bool ok = true;
+            for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++k) {
+                const uint32_t acc = tmem + (uint32_t)((k & 1) * a.zt * NB);
+                ok = mbar_wait_role(&b_accfree[k & 1], (uint32_t)((k >> 1) & 1) ^ 1u, &s_abort, a.err);
+                if (!ok) break;
+                for (int cb = 0; cb < ncb; ++cb) {
+                    ok = mbar_wait_role(&b_full[st], ph, &s_abort, a.err) &&
+                         mbar_wait_role(&b_wfull[st], ph, &s_abort, a.err);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t wbase = base + (uint32_t)st * stage_bytes, hbase = wbase + kWBytes;
+                    for (int zi = 0; zi < a.zt + 2; ++zi) {
+                        const int lo = max(0, zi - 2), nw = min(a.zt - 1, zi) - lo + 1;
+                        const uint32_t d = acc + (uint32_t)(lo * NB);
+                        const uint64_t ad0 = smem_desc(hbase + (uint32_t)(zi * kPlaneBytes), kHX * 16, 2 * kHX * 16);
+                        const uint64_t bd0 =
+                            smem_desc(wbase + (uint32_t)((lo - (zi - 2)) * NB * 32), 8 * 16, 2 * 8 * 16);
+                        const uint32_t id = idesc_bf16(128, nw * NB);
+                        // the newest output plane of the window starts at its first tap
+                        const bool start = cb == 0 && zi < a.zt;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            float a = v[e] + (bias ? bias[c0 + e] : 0.f);
-                            if (relu) a = fmaxf(a, 0.f);
-                            o[e] = __float2bfloat16(a);
+                        for (int t = 0; t < 9; ++t) {
+                            // start addresses are in 16-byte units in the low bits of the descriptors
+                            const uint64_t ad = ad0 + (uint64_t)((t / 3) * 2 * kHX + t % 3);
+                            const uint64_t bd = bd0 + (uint64_t)(t * 6 * NB);
+                            if (t == 0 && start) {
+                                if (nw > 1) tc_mma(d, ad, bd, idesc_bf16(128, (nw - 1) * NB), 1u);
+                                tc_mma(d + (uint32_t)((nw - 1) * NB), ad, bd + (uint64_t)((nw - 1) * 2 * NB),
+                                       idesc_bf16(128, NB), 0u);
+                            } else {
+                                tc_mma(d, ad, bd, id, 1u);
+                            }
                         }
+                    }
+                    tc_commit(&b_empty[st]);
+                    if (++st == a.nstage) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (ok) tc_commit(&b_acc[k & 1]);
+            }
+            tc_commit(&b_end);
+            if (!mbar_drain(&b_end, 0u)) atomicMax(a.err, 2);
+        }
+        __syncwarp();
+    } else {
+        // ---- read-out ----
+        const int m = warp * 32 + lane;
+        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        int k = 0;
+        for (int item = blockIdx.x; item < items; item += gridDim.x, ++k) {
+            int x0, y0, z0, blk;
+            origin(item, x0, y0, z0, blk);
+            const int gx = x0 + (m & 7), gy = y0 + (m >> 3);
+            const bool in2 = gx < g.nx && gy < g.ny;
+            if (!mbar_wait_role(&b_acc[k & 1], (uint32_t)((k >> 1) & 1), &s_abort, a.err)) break;
+            __syncwarp();
+            tc_fence_after();
+            const uint32_t acc = lane_base + (uint32_t)((k & 1) * a.zt * NB);
+            for (int j = 0; j < a.zt && z0 + j < g.nz; ++j) {
+                bf16* orow = a.out + ((size_t)((long)(z0 + j) * g.ny + (in2 ? gy : 0)) * g.nx + (in2 ? gx : 0)) * a.N +
+                             blk * NB;
+#pragma unroll
+                for (int c0 = 0; c0 < NB; c0 += 16) {
+                    uint32_t r[16];
+                    tmem_ld16_issue(acc + (uint32_t)(j * NB + c0), r);
+                    float bv[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) bv[e] = a.bias ? __ldg(a.bias + blk * NB + c0 + e) : 0.f;
+                    tmem_ld_wait();
+                    __align__(16) bf16 o[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        float v = __uint_as_float(r[e]) + bv[e];
+                        if (a.relu) v = fmaxf(v, 0.f);
+                        o[e] = __float2bfloat16(v);
+                    }
+                    if (in2) {
                         *reinterpret_cast<uint4*>(orow + c0) = *reinterpret_cast<const uint4*>(o);
+                        *reinterpret_cast<uint4*>(orow + c0 + 8) = *reinterpret_cast<const uint4*>(o + 8);
                     }
                 }
             }
             tc_fence_before();
+            mbar_arrive(&b_accfree[k & 1]);
         }
     }
-    // outstanding copies and MMAs (bounded) before TMEM is released; a phase
-    // whose wait gave up must be seen complete before the dealloc
-    cp_async_wait_all();
-    for (int b = 0; b < 2; ++b) wait_mma(b);
-    for (int b = 0; b < 2; ++b)
-        if (unconfirmed[b] && !mbar_drain(&mbar[b], uphase[b])) atomicMax(err, 2);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+    if (warp == kZbMmaWarp)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.ncols) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -904,7 +1014,8 @@ struct cdi_unet {
     // parameters
     float *W[kLayers], *B[kLayers], *gW[kLayers], *gB[kLayers];
     float *mW[kLayers], *vW[kLayers], *mB[kLayers], *vB[kLayers];
-    bf16 *Wb[kLayers], *Wt[kLayers];
+    bf16 *Wb[kLayers], *Wt[kLayers];    // weights of the mma.sync kernels
+    bf16 *Wk[kLayers], *Wkt[kLayers];   // weights of the tcgen05 convolution (forward, data gradient)
     int ci_pad[kLayers], co_pad[kLayers];
     // activations and gradients (BF16, channels last)
     bf16 *x, *e0, *p0, *e1, *p1, *e2, *p2, *b, *c2, *d2, *c1, *d1, *c0, *d0;
@@ -979,6 +1090,8 @@ void unet_carve(cdi_unet* u, char* base, size_t* total) {
         const size_t np = (size_t)kTaps[l] * u->ci_pad[l] * u->co_pad[l];
         u->Wb[l] = (bf16*)cv.take(np * 2);
         u->Wt[l] = (bf16*)cv.take(np * 2);
+        u->Wk[l] = (bf16*)cv.take(np * 2);
+        u->Wkt[l] = (bf16*)cv.take(np * 2);
     }
     const long N0 = u->g[0].N, N1 = u->g[1].N, N2 = u->g[2].N, N3 = u->g[3].N;
     auto act = [&](long n, int c) { return (bf16*)cv.take((size_t)n * c * 2); };
@@ -1026,38 +1139,73 @@ void unet_carve(cdi_unet* u, char* base, size_t* total) {
     *total = cv.off + 256;
 }
 
-// tcgen05 convolution launch: a persistent grid of as many CTAs as fit at once (shared memory
-// bounds the CTAs per SM below what the TMEM columns allow, so no TMEM allocation ever waits)
-void conv_tc(cdi_unet* u, const CG& gl, const bf16* in, int cin, const bf16* w, int N, const float* bias, int cout,
-             bf16* out, int out_stride, bool relu, const bf16* up = nullptr, int cup = 0) {
-    static int nsm = 0, smem_sm = 0;
-    static bool attr = false;
-    const int ncols = 2 * N <= 32 ? 32 : 2 * N <= 64 ? 64 : 2 * N <= 128 ? 128 : 2 * N <= 256 ? 256 : 512;
-    const size_t smem = 2 * (size_t)kHaloBytes + kGuardBytes + 2 * (size_t)kTapsPerIter * 2 * N * 16;
-    if (!attr) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        attr = true;
+// Planes of a tile of the tcgen05 convolution.  More planes share each staged halo plane and fill the
+// MMAs' N (planes 2 .. zt-1 of a tile feed three output planes at once), fewer give more tiles to spread
+// over the SMs.  Takes the zt of least estimated cycles: rounds of the persistent grid times the MMA cycles
+// of a tile (32 cycles of A and NB / 4 of B a column block, or NB / 2 of arithmetic, whichever is larger)
+// plus 2500 for staging and reading out its ends.  NB zt <= 256 (two accumulator sets in 512 columns).
+int conv_planes(const CG& g, int NB, int nblk, int ncb, int nsm) {
+    const int cap = std::min(8, 256 / NB);
+    long best = 0;
+    int zt_best = 1;
+    for (int zt = 1; zt <= cap; zt *= 2) {
+        if (zt > 1 && zt / 2 >= g.nz) break;
+        const long items = (long)((g.nx + kTileX - 1) / kTileX) * ((g.ny + kTileY - 1) / kTileY) *
+                           ((g.nz + zt - 1) / zt) * nblk;
+        long cyc = 0;
+        for (int zi = 0; zi < zt + 2; ++zi) {
+            const int nw = std::min(zt - 1, zi) - std::max(0, zi - 2) + 1;
+            cyc += std::max(32 + nw * NB / 4, nw * NB / 2);
+        }
+        const long cost = (items + nsm - 1) / nsm * (9 * cyc * ncb + 2500);
+        if (zt == 1 || cost < best) {
+            best = cost;
+            zt_best = zt;
+        }
     }
-    // CTAs per SM: shared memory (1 KB reserved per CTA, plus the static 1 KB), threads, TMEM columns
-    int per = (int)((size_t)smem_sm / (smem + 2048));
-    per = std::max(1, std::min({per, 2048 / kTcThreads, 512 / ncols}));
-    const long tiles = (long)((gl.nx + kTileX - 1) / kTileX) * ((gl.ny + kTileY - 1) / kTileY) *
-                       ((gl.nz + kTileZ - 1) / kTileZ);
-    const unsigned grid = (unsigned)std::max(1L, std::min(tiles, (long)nsm * per));
-    k_conv_tc<<<grid, kTcThreads, smem, u->stream>>>(gl, in, cin, up, cup, w, N, bias, cout, out, out_stride,
-                                                     relu ? 1 : 0, ncols, u->tc_err);
+    return zt_best;
+}
+
+constexpr size_t kConvSmem = 220 * 1024;  // of the 227 KB a CTA may use
+
+template <int NB>
+void conv_zb(const ConvArgs& a, size_t smem, unsigned grid, cudaStream_t s) {
+    cudaFuncSetAttribute(k_conv_zb<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
+    k_conv_zb<NB><<<grid, kZbThreads, smem, s>>>(a);
+}
+
+// tcgen05 convolution launch: a persistent grid of one CTA per SM (its shared memory lets no second one in,
+// so no TMEM allocation waits for another CTA of the launch)
+void conv_tc(cdi_unet* u, const CG& gl, const bf16* in, int cin, const bf16* w, int N, const float* bias, bf16* out,
+             bool relu, const bf16* up = nullptr, int cup = 0) {
+    int dev = 0, nsm = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int NB = conv_nb(N);
+    ConvArgs a{gl, in, up, cin, cup, w, bias, out, N, relu ? 1 : 0, 0, 0, N / NB, 0, u->tc_err};
+    a.zt = conv_planes(gl, NB, a.nblk, cin / 16, nsm);
+    const size_t stage = (size_t)27 * 32 * NB + (size_t)(a.zt + 2) * kPlaneBytes;
+    a.nstage = (int)std::min<size_t>(kZbMaxStages, kConvSmem / stage);
+    a.ncols = 32;
+    while (a.ncols < 2 * a.zt * NB) a.ncols *= 2;
+    const long items = (long)((gl.nx + kTileX - 1) / kTileX) * ((gl.ny + kTileY - 1) / kTileY) *
+                       ((gl.nz + a.zt - 1) / a.zt) * a.nblk;
+    const unsigned grid = (unsigned)std::min<long>(items, nsm);
+    // more than half of an SM's shared memory, so one CTA per SM whatever the stages need
+    const size_t smem = std::max(a.nstage * stage, (size_t)116 * 1024);
+    switch (NB) {
+        case 16: conv_zb<16>(a, smem, grid, u->stream); break;
+        case 32: conv_zb<32>(a, smem, grid, u->stream); break;
+        case 48: conv_zb<48>(a, smem, grid, u->stream); break;
+        default: conv_zb<64>(a, smem, grid, u->stream); break;
+    }
 }
 
 // y = conv(in) for layer l on level grid gl into out (stride, offset)
 template <bool OUTF32>
 void conv_fwd(cdi_unet* u, int l, const CG& gl, const bf16* in, void* out, int stride, int off, bool relu) {
     if (!OUTF32 && kTaps[l] == 27 && u->use_tc && off == 0 && stride == u->co_pad[l]) {
-        conv_tc(u, gl, in, u->ci_pad[l], u->Wb[l], u->co_pad[l], u->B[l], u->co_pad[l], (bf16*)out, stride, relu);
+        conv_tc(u, gl, in, u->ci_pad[l], u->Wk[l], u->co_pad[l], u->B[l], (bf16*)out, relu);
         return;
     }
     const unsigned gb = (unsigned)((gl.N + 63) / 64);
@@ -1082,7 +1230,7 @@ void conv_fwd(cdi_unet* u, int l, const CG& gl, const bf16* in, void* out, int s
 // dx (BF16 [N][ci_pad]) = adjoint of layer l applied to dy (BF16 [N][co_pad])
 void conv_dgrad(cdi_unet* u, int l, const CG& gl, const bf16* dy, bf16* dx) {
     if (kTaps[l] == 27 && u->use_tc) {
-        conv_tc(u, gl, dy, u->co_pad[l], u->Wt[l], u->ci_pad[l], nullptr, u->ci_pad[l], dx, u->ci_pad[l], false);
+        conv_tc(u, gl, dy, u->co_pad[l], u->Wkt[l], u->ci_pad[l], nullptr, dx, false);
         return;
     }
     const unsigned gb = (unsigned)((gl.N + 63) / 64);
@@ -1153,7 +1301,7 @@ void refresh_weights(cdi_unet* u) {
     for (int l = 0; l < kLayers; ++l) {
         const long n = (long)kTaps[l] * u->co_pad[l] * u->ci_pad[l];
         k_weights_bf16<<<blocks(n), 256, 0, u->stream>>>(u->W[l], kTaps[l], kCout[l], kCin[l], u->co_pad[l],
-                                                          u->ci_pad[l], u->Wb[l], u->Wt[l]);
+                                                          u->ci_pad[l], u->Wb[l], u->Wt[l], u->Wk[l], u->Wkt[l]);
     }
     u->weights_ready = true;
 }
@@ -1174,9 +1322,9 @@ void forward(cdi_unet* u, bool keep_concat = true) {
     conv_fwd<false>(u, 3, g[3], u->p2, u->b, 128, 0, true);
     g_launches += 7;
     if (fuse) {
-        conv_tc(u, g[2], u->e2, 192, u->Wb[4], 64, u->B[4], 64, u->d2, 64, true, u->b, 128);
-        conv_tc(u, g[1], u->e1, 96, u->Wb[5], 32, u->B[5], 32, u->d1, 32, true, u->d2, 64);
-        conv_tc(u, g[0], u->e0, 48, u->Wb[6], 16, u->B[6], 16, u->d0, 16, true, u->d1, 32);
+        conv_tc(u, g[2], u->e2, 192, u->Wk[4], 64, u->B[4], u->d2, true, u->b, 128);
+        conv_tc(u, g[1], u->e1, 96, u->Wk[5], 32, u->B[5], u->d1, true, u->d2, 64);
+        conv_tc(u, g[0], u->e0, 48, u->Wk[6], 16, u->B[6], u->d0, true, u->d1, 32);
         g_launches += 3;
     } else {
         k_up<<<blocks(g[2].N * 16L), 256, 0, s>>>(g[2], u->b, 128, u->c2, 192, 0);
