@@ -339,18 +339,39 @@ __global__ void k_weights_bf16(const float* W, int taps, int cout, int cin, int 
     }
 }
 
-__global__ void k_input_host(int N, const double* x2, bf16* x) {  // x2: [N][2] from the host
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)N * 16) return;
-    const int c = (int)(t % 16), v = (int)(t / 16);
-    x[t] = __float2bfloat16(c < 2 ? (float)x2[(size_t)v * 2 + c] : 0.f);
+// network input in two forms: pairs xp [N][2] for the first layer's tcgen05 convolution and, where x is not null,
+// padded to 16 channels for the mma.sync kernels and the weight gradient
+__device__ __forceinline__ void put_input(int v, float a, float b, bf16* xp, bf16* x) {
+    const unsigned p = pack2(__float2bfloat16(a), __float2bfloat16(b));
+    reinterpret_cast<unsigned*>(xp)[v] = p;
+    if (x) {
+        uint4* q = reinterpret_cast<uint4*>(x + (size_t)v * 16);
+        q[0] = make_uint4(p, 0u, 0u, 0u);
+        q[1] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+__global__ void k_input_host(int N, const double* x2, bf16* xp, bf16* x) {  // x2: [N][2] from the host
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < N) put_input(v, (float)x2[(size_t)v * 2], (float)x2[(size_t)v * 2 + 1], xp, x);
 }
 
-__global__ void k_input_dev(int N, const float* x2, bf16* x) {  // x2: [N][2] on the device
+__global__ void k_input_dev16(int N, const float* x2, bf16* xp, bf16* x) {
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < N) put_input(v, x2[(size_t)v * 2], x2[(size_t)v * 2 + 1], xp, x);
+}
+
+// x2: [N][2] on the device (4-byte aligned), N even; two voxels a thread.  The 16-channel form it replaces wrote
+// 32 bytes a voxel, a channel a thread (615 us at 256^3).
+__global__ void k_input_dev(int N, const float* x2, bf16* xp) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)N * 16) return;
-    const int c = (int)(t % 16), v = (int)(t / 16);
-    x[t] = __float2bfloat16(c < 2 ? x2[(size_t)v * 2 + c] : 0.f);
+    if (2 * t >= N) return;
+    const float* q = x2 + 4 * t;
+    const bool al = (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+    const float4 v = al ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
+    uint2 o;
+    o.x = pack2(__float2bfloat16(v.x), __float2bfloat16(v.y));
+    o.y = pack2(__float2bfloat16(v.z), __float2bfloat16(v.w));
+    reinterpret_cast<uint2*>(xp)[t] = o;
 }
 
 // scales of one prediction from ||f||_2 (one thread): sd = {1/rms(f), rms(f) max(rho) h^2}
@@ -367,18 +388,13 @@ __global__ void k_solver_scales(const double* fnorm, int N, double rho_h2, doubl
 // form; removed here with the double-float mean in the FP32-mixed form) and phi
 template <typename T>
 __global__ void k_input_solver(int N, const FT<T>* f, const float* fmean_df, const T* phi, float drho, float rho2,
-                               float inv_rmax, const double* sd, const float* sf, bf16* x) {
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)N * 16) return;
-    const int c = (int)(t % 16), v = (int)(t / 16);
-    float val = 0.f;
-    if (c == 0) {
-        if constexpr (sizeof(T) == 8) val = (float)(f[v] * sd[0]);
-        else val = ((f[v] - fmean_df[0]) - fmean_df[1]) * sf[0];
-    } else if (c == 1) {
-        val = (drho * (float)phi[v] + rho2) * inv_rmax;
-    }
-    x[t] = __float2bfloat16(val);
+                               float inv_rmax, const double* sd, const float* sf, bf16* xp, bf16* x) {
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= N) return;
+    float val;
+    if constexpr (sizeof(T) == 8) val = (float)(f[v] * sd[0]);
+    else val = ((f[v] - fmean_df[0]) - fmean_df[1]) * sf[0];
+    put_input(v, val, (drho * (float)phi[v] + rho2) * inv_rmax, xp, x);
 }
 
 template <typename T>
@@ -416,6 +432,13 @@ unsigned blocks(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 // weight rows, stored in the order dz = +1, 0, -1.  Every accumulator still
 // receives its products in the order channel block, dz, dy, dx.
 //
+// The first layer has two input channels (PAIRS): its rows are staged as one
+// 16-byte unit a voxel, 4 bytes of it copied and the rest zero, and the second
+// half of K reads a block of zeros.  (Packing dx and dy into K would need two
+// MMAs a plane instead of nine, but sums the products in another order: the
+// BF16 roundings that flip then, about one in 10^6, grow through the layers
+// to the rounding noise of the whole network, 1e-3 of the output.)
+//
 // Roles: warps 0-3 read the accumulators of a finished tile (bias, ReLU, BF16
 // rounding, 16-byte stores), warp 4 issues the MMAs (one thread), warps 5-7
 // stage the input with cp.async, one thread of them the weights with one bulk
@@ -423,16 +446,26 @@ unsigned blocks(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 // so copies, MMAs and read-out of consecutive tiles overlap.  zt is chosen by
 // conv_planes (below).
 //
-// Measured, forward pass of the network (GB300): 256^3 8.05 -> 3.50 ms, 128^3
-// 1.20 -> 0.52 ms, 40 x 24 x 16 283 -> 107 us against one MMA of N = NB a tap
-// and plane with a CTA barrier every 18 MMAs; bit-identical.
+// Measured, forward pass of the network (GB300): 256^3 8.05 -> 2.07 ms (650
+// TFLOP/s), 128^3 1.20 -> 0.34 ms, 40 x 24 x 16 283 -> 102 us against one MMA
+// of N = NB a tap and plane with a CTA barrier every 18 MMAs, an input kernel
+// of 32 bytes a voxel (615 us at 256^3, now 31) and a separate head (396 us,
+// now in the last layer's read-out, whose output is not stored).  The three
+// dz taps in N alone gave 3.50 ms; handing a stage over as soon as its copies
+// land, instead of after the next stage's have been issued, 460 -> 311 us on
+// the 96 -> 32 layer at 128^3.
 // ---------------------------------------------------------------------------
 constexpr int kZbThreads = 256, kZbProd = 96, kZbMmaWarp = 4;
 constexpr int kTileX = 8, kTileY = 16;
 constexpr int kHX = kTileX + 2, kHY = kTileY + 2;
 constexpr int kPlaneUnits = kHY * 2 * kHX;       // 16-byte units of one staged plane: [y][8-channel half][x]
-constexpr int kPlaneBytes = kPlaneUnits * 16;
 constexpr int kZbMaxStages = 4;
+// PAIRS: 16-byte units of a plane [y][x], and the block of zeros (with the same row stride) of channels 8..15
+constexpr int kPairUnits = kHY * kHX, kPairZeroBytes = kTileY * kHX * 16;
+
+// bytes of one stage's weights and of one staged plane
+__host__ __device__ constexpr uint32_t zb_wbytes(int NB) { return 27u * 32u * NB; }
+__host__ __device__ constexpr uint32_t zb_plane(bool pairs) { return 16u * (pairs ? kPairUnits : kPlaneUnits); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -443,6 +476,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
@@ -519,18 +561,35 @@ __device__ __forceinline__ void cp_async16(uint32_t saddr, const void* g, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr), "l"(g), "r"(valid ? 16 : 0)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async4(uint32_t saddr, const void* g, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(saddr), "l"(g), "r"(valid ? 4 : 0) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// 16 consecutive FP32 columns of this thread's TMEM lane (no wait)
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
+// 16 (and, from a second place, 16 more) consecutive FP32 columns of this thread's TMEM lane, complete on return
+#define TM_OUT16(r, o)                                                                                            \
+    "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]),    \
+        "=r"(r[o + 7]), "=r"(r[o + 8]), "=r"(r[o + 9]), "=r"(r[o + 10]), "=r"(r[o + 11]), "=r"(r[o + 12]),         \
+        "=r"(r[o + 13]), "=r"(r[o + 14]), "=r"(r[o + 15])
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : TM_OUT16(r, 0)
+        : "r"(taddr)
+        : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+        "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : TM_OUT16(r, 0), TM_OUT16(r, 16)
+        : "r"(taddr)
+        : "memory");
+}
+#undef TM_OUT16
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -562,12 +621,15 @@ __device__ __forceinline__ bool mbar_wait_role(uint64_t* bar, uint32_t parity, v
 
 struct ConvArgs {
     CG g;
-    const bf16* in;     // [voxel][cin - cup]
+    const bf16* in;     // [voxel][cin - cup]; PAIRS: [voxel][2]
     const bf16* up;     // coarse input of the first cup channels (nearest upsampling of half the extents), or null
     int cin, cup;       // multiples of 16
     const bf16* w;      // blocked weights (k_weights_bf16): [channel block of NB][16 input channels][9][3 NB][16]
     const float* bias;  // [N] or null
-    bf16* out;          // [voxel][N]
+    bf16* out;          // [voxel][N], or null (NB = 16 with the head only)
+    const bf16* head_w;   // NB = 16: also y[voxel] = head_b + sum_c head_w[c] (this layer's BF16 output c), or null
+    const float* head_b;
+    float* y;
     int N, relu;
     int zt, nstage, nblk, ncols;  // planes of a tile, staging buffers, N / NB, TMEM columns (a power of two >= 2 zt NB)
     int* err;
@@ -578,8 +640,8 @@ struct ConvArgs {
 // issued has been seen complete (a last commit, waited for with a poll bound); if that wait runs out too,
 // *err is set to 2 (the CTA must still release its columns before it exits, so their contents are not to
 // be trusted by any later kernel of the context).
-template <int NB>
-__global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
+template <int NB, bool PAIRS>
+__global__ void __launch_bounds__(kZbThreads, PAIRS ? 2 : 1) k_conv_zb(const ConvArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t b_full[kZbMaxStages], b_wfull[kZbMaxStages], b_empty[kZbMaxStages];
     __shared__ __align__(8) uint64_t b_acc[2], b_accfree[2], b_end;
@@ -587,8 +649,8 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
     __shared__ volatile int s_abort;
     const CG& g = a.g;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr uint32_t kWBytes = 27u * 32u * NB;
-    const uint32_t stage_bytes = kWBytes + (uint32_t)((a.zt + 2) * kPlaneBytes);
+    constexpr uint32_t kWBytes = zb_wbytes(NB), kPlane = zb_plane(PAIRS);
+    const uint32_t stage_bytes = kWBytes + (uint32_t)(a.zt + 2) * kPlane;
     const uint32_t base = smem_u32(smem);
 
     if (warp == kZbMmaWarp) {
@@ -610,6 +672,12 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
         mbar_init(&b_end, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (PAIRS) {  // the rows' other channels and the block of zeros after the stages stay zero
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        uint4* q = reinterpret_cast<uint4*>(smem);
+        for (int i = tid; i < (int)(a.nstage * stage_bytes + kPairZeroBytes) / 16; i += kZbThreads) q[i] = z;
+        fence_proxy_async();
     }
     tc_fence_before();
     __syncthreads();
@@ -649,6 +717,19 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
                     bulk_load(wbase, a.w + (size_t)(blk * ncb + cb) * (kWBytes / 2), kWBytes, &b_wfull[st]);
                     ++issued;
                 }
+                if (PAIRS) {
+                    for (int u = pt; u < kPairUnits; u += kZbProd) {
+                        const int hy = u / kHX, gx = x0 + (u - hy * kHX) - 1, gy = y0 + hy - 1;
+                        const bool in2 = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny;
+                        const bf16* p = a.in + (in2 ? 2 * ((long)gy * g.nx + gx) : 0);
+                        uint32_t dst = hbase + (uint32_t)u * 16u;
+                        for (int hz = 0; hz < a.zt + 2; ++hz, dst += kPlane) {
+                            const int gz = z0 + hz - 1;
+                            const bool in3 = in2 && gz >= 0 && gz < g.nz;
+                            cp_async4(dst, in3 ? p + 2 * (long)gz * g.nx * g.ny : a.in, in3);
+                        }
+                    }
+                } else {
                 const bool isup = cb * 16 < a.cup;
                 const int sh = isup ? 1 : 0, C = isup ? a.cup : a.cin - a.cup;
                 const int snx = g.nx >> sh, sny = g.ny >> sh;
@@ -660,11 +741,12 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
                     const bool in2 = gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny;
                     const bf16* p = src0 + (in2 ? ((size_t)(gy >> sh) * snx + (gx >> sh)) * C : 0) + kc * 8;
                     uint32_t dst = hbase + (uint32_t)((hy * 2 + kc) * kHX + hx) * 16u;
-                    for (int hz = 0; hz < a.zt + 2; ++hz, dst += kPlaneBytes) {
+                    for (int hz = 0; hz < a.zt + 2; ++hz, dst += kPlane) {
                         const int gz = z0 + hz - 1;
                         const bool in3 = in2 && gz >= 0 && gz < g.nz;
                         cp_async16(dst, in3 ? p + (size_t)(gz >> sh) * zstride : a.in, in3);
                     }
+                }
                 }
                 cp_async_commit();
                 // hand over the stage before this one: its copies are done when at most one group is open
@@ -677,6 +759,13 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
                 if (++st == a.nstage) {
                     st = 0;
                     ph ^= 1u;
+                }
+                // and this one at once where the next buffer is not free yet
+                if (!mbar_test_wait(&b_empty[st], ph)) {
+                    cp_async_wait_all();
+                    fence_proxy_async();
+                    mbar_arrive(prev);
+                    prev = nullptr;
                 }
             }
         }
@@ -695,6 +784,7 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
             int st = 0, k = 0;
             uint32_t ph = 0u;
             bool ok = true;
+            const uint32_t zeros = base + (uint32_t)a.nstage * stage_bytes;  // PAIRS
             for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++k) {
                 const uint32_t acc = tmem + (uint32_t)((k & 1) * a.zt * NB);
                 ok = mbar_wait_role(&b_accfree[k & 1], (uint32_t)((k >> 1) & 1) ^ 1u, &s_abort, a.err);
@@ -708,7 +798,8 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
                     for (int zi = 0; zi < a.zt + 2; ++zi) {
                         const int lo = max(0, zi - 2), nw = min(a.zt - 1, zi) - lo + 1;
                         const uint32_t d = acc + (uint32_t)(lo * NB);
-                        const uint64_t ad0 = smem_desc(hbase + (uint32_t)(zi * kPlaneBytes), kHX * 16, 2 * kHX * 16);
+                        const uint32_t pl = hbase + (uint32_t)zi * kPlane;
+                        const uint64_t ad0 = smem_desc(pl, kHX * 16, 2 * kHX * 16);
                         const uint64_t bd0 =
                             smem_desc(wbase + (uint32_t)((lo - (zi - 2)) * NB * 32), 8 * 16, 2 * 8 * 16);
                         const uint32_t id = idesc_bf16(128, nw * NB);
@@ -717,7 +808,9 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
 #pragma unroll
                         for (int t = 0; t < 9; ++t) {
                             // start addresses are in 16-byte units in the low bits of the descriptors
-                            const uint64_t ad = ad0 + (uint64_t)((t / 3) * 2 * kHX + t % 3);
+                            const uint32_t tp = pl + (uint32_t)((t / 3) * kHX + t % 3) * 16u;
+                            const uint64_t ad = PAIRS ? smem_desc(tp, zeros - tp, kHX * 16)
+                                                      : ad0 + (uint64_t)((t / 3) * 2 * kHX + t % 3);
                             const uint64_t bd = bd0 + (uint64_t)(t * 6 * NB);
                             if (t == 0 && start) {
                                 if (nw > 1) tc_mma(d, ad, bd, idesc_bf16(128, (nw - 1) * NB), 1u);
@@ -744,6 +837,16 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
         // ---- read-out ----
         const int m = warp * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        // NB = 16: one channel block, so its biases and the head's weights stay in registers
+        float bias0[16], head[16], hbias = 0.f;
+        if (NB == 16) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                bias0[e] = a.bias ? a.bias[e] : 0.f;
+                head[e] = a.y ? __bfloat162float(a.head_w[e]) : 0.f;
+            }
+            if (a.y) hbias = a.head_b[0];
+        }
         int k = 0;
         for (int item = blockIdx.x; item < items; item += gridDim.x, ++k) {
             int x0, y0, z0, blk;
@@ -754,27 +857,34 @@ __global__ void __launch_bounds__(kZbThreads, 1) k_conv_zb(const ConvArgs a) {
             __syncwarp();
             tc_fence_after();
             const uint32_t acc = lane_base + (uint32_t)((k & 1) * a.zt * NB);
-            for (int j = 0; j < a.zt && z0 + j < g.nz; ++j) {
-                bf16* orow = a.out + ((size_t)((long)(z0 + j) * g.ny + (in2 ? gy : 0)) * g.nx + (in2 ? gx : 0)) * a.N +
-                             blk * NB;
+            const size_t v0 = in2 ? ((size_t)z0 * g.ny + gy) * g.nx + gx : 0;
+            const int chunks = min(a.zt, g.nz - z0) * (NB / 16);
+            for (int q0 = 0; q0 < chunks; q0 += 2) {  // 16 columns each, two at a time
+                uint32_t r[32];
+                if (q0 + 1 < chunks) tmem_ld32(acc + (uint32_t)(q0 * 16), r);
+                else tmem_ld16(acc + (uint32_t)(q0 * 16), r);
 #pragma unroll
-                for (int c0 = 0; c0 < NB; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld16_issue(acc + (uint32_t)(j * NB + c0), r);
-                    float bv[16];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) bv[e] = a.bias ? __ldg(a.bias + blk * NB + c0 + e) : 0.f;
-                    tmem_ld_wait();
+                for (int h = 0; h < 2; ++h) {
+                    const int q = q0 + h, j = q / (NB / 16), c0 = (q - j * (NB / 16)) * 16 + blk * NB;
+                    if (q >= chunks || !in2) continue;
+                    const size_t v = v0 + (size_t)j * g.nx * g.ny;
                     __align__(16) bf16 o[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        float v = __uint_as_float(r[e]) + bv[e];
-                        if (a.relu) v = fmaxf(v, 0.f);
-                        o[e] = __float2bfloat16(v);
+                        float x = __uint_as_float(r[16 * h + e]) + (NB == 16 ? bias0[e] : a.bias ? __ldg(a.bias + c0 + e) : 0.f);
+                        if (a.relu) x = fmaxf(x, 0.f);
+                        o[e] = __float2bfloat16(x);
                     }
-                    if (in2) {
-                        *reinterpret_cast<uint4*>(orow + c0) = *reinterpret_cast<const uint4*>(o);
-                        *reinterpret_cast<uint4*>(orow + c0 + 8) = *reinterpret_cast<const uint4*>(o + 8);
+                    if (NB > 16 || a.out) {
+                        bf16* orow = a.out + v * a.N + c0;
+                        *reinterpret_cast<uint4*>(orow) = *reinterpret_cast<const uint4*>(o);
+                        *reinterpret_cast<uint4*>(orow + 8) = *reinterpret_cast<const uint4*>(o + 8);
+                    }
+                    if (NB == 16 && a.y) {
+                        float sum = 0.f;
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) sum = fmaf(__bfloat162float(o[e]), head[e], sum);
+                        a.y[v] = sum + hbias;
                     }
                 }
             }
@@ -1018,6 +1128,7 @@ struct cdi_unet {
     bf16 *Wk[kLayers], *Wkt[kLayers];   // weights of the tcgen05 convolution (forward, data gradient)
     int ci_pad[kLayers], co_pad[kLayers];
     // activations and gradients (BF16, channels last)
+    bf16 *xp;  // input pairs [N][2]
     bf16 *x, *e0, *p0, *e1, *p1, *e2, *p2, *b, *c2, *d2, *c1, *d1, *c0, *d0;
     bf16 *gy, *gd0, *gc0, *gd1, *gc1, *gd2, *gc2, *gb, *gp2, *ge2, *gp1, *ge1, *gp0, *ge0;
     float *y, *t, *part;
@@ -1096,6 +1207,7 @@ void unet_carve(cdi_unet* u, char* base, size_t* total) {
     const long N0 = u->g[0].N, N1 = u->g[1].N, N2 = u->g[2].N, N3 = u->g[3].N;
     auto act = [&](long n, int c) { return (bf16*)cv.take((size_t)n * c * 2); };
     u->x = act(N0, 16);
+    u->xp = act(N0, 2);
     u->e0 = act(N0, 16);
     u->p0 = act(N1, 16);
     u->e1 = act(N1, 32);
@@ -1168,37 +1280,60 @@ int conv_planes(const CG& g, int NB, int nblk, int ncb, int nsm) {
 
 constexpr size_t kConvSmem = 220 * 1024;  // of the 227 KB a CTA may use
 
-template <int NB>
+template <int NB, bool PAIRS = false>
 void conv_zb(const ConvArgs& a, size_t smem, unsigned grid, cudaStream_t s) {
-    cudaFuncSetAttribute(k_conv_zb<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
-    k_conv_zb<NB><<<grid, kZbThreads, smem, s>>>(a);
+    cudaFuncSetAttribute(k_conv_zb<NB, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
+    k_conv_zb<NB, PAIRS><<<grid, kZbThreads, smem, s>>>(a);
 }
 
-// tcgen05 convolution launch: a persistent grid of one CTA per SM (its shared memory lets no second one in,
-// so no TMEM allocation waits for another CTA of the launch)
-void conv_tc(cdi_unet* u, const CG& gl, const bf16* in, int cin, const bf16* w, int N, const float* bias, bf16* out,
-             bool relu, const bf16* up = nullptr, int cup = 0) {
+// launch of the tcgen05 convolution of the layer a describes (all but its split): a persistent grid of one CTA per
+// SM, or two for PAIRS, whose shared memory lets no more in, so no TMEM allocation waits for another CTA of the launch
+void conv_launch(ConvArgs a, bool pairs, cudaStream_t s) {
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int NB = conv_nb(N);
-    ConvArgs a{gl, in, up, cin, cup, w, bias, out, N, relu ? 1 : 0, 0, 0, N / NB, 0, u->tc_err};
-    a.zt = conv_planes(gl, NB, a.nblk, cin / 16, nsm);
-    const size_t stage = (size_t)27 * 32 * NB + (size_t)(a.zt + 2) * kPlaneBytes;
-    a.nstage = (int)std::min<size_t>(kZbMaxStages, kConvSmem / stage);
+    const int per = pairs ? 2 : 1;
+    const int NB = conv_nb(a.N);
+    a.nblk = a.N / NB;
+    a.zt = conv_planes(a.g, NB, a.nblk, a.cin / 16, nsm * per);
+    const size_t stage = zb_wbytes(NB) + (size_t)(a.zt + 2) * zb_plane(pairs);
+    const size_t extra = pairs ? kPairZeroBytes : 0;
+    a.nstage = (int)std::min<size_t>(kZbMaxStages, (kConvSmem / per - extra - (per - 1) * 2048) / stage);
     a.ncols = 32;
     while (a.ncols < 2 * a.zt * NB) a.ncols *= 2;
-    const long items = (long)((gl.nx + kTileX - 1) / kTileX) * ((gl.ny + kTileY - 1) / kTileY) *
-                       ((gl.nz + a.zt - 1) / a.zt) * a.nblk;
-    const unsigned grid = (unsigned)std::min<long>(items, nsm);
-    // more than half of an SM's shared memory, so one CTA per SM whatever the stages need
-    const size_t smem = std::max(a.nstage * stage, (size_t)116 * 1024);
-    switch (NB) {
-        case 16: conv_zb<16>(a, smem, grid, u->stream); break;
-        case 32: conv_zb<32>(a, smem, grid, u->stream); break;
-        case 48: conv_zb<48>(a, smem, grid, u->stream); break;
-        default: conv_zb<64>(a, smem, grid, u->stream); break;
+    const long items = (long)((a.g.nx + kTileX - 1) / kTileX) * ((a.g.ny + kTileY - 1) / kTileY) *
+                       ((a.g.nz + a.zt - 1) / a.zt) * a.nblk;
+    const unsigned grid = (unsigned)std::min<long>(items, (long)nsm * per);
+    // at least what keeps another CTA out of the SM
+    const size_t smem = std::max(a.nstage * stage + extra, (size_t)(pairs ? 78 : 116) * 1024);
+    if (pairs) {
+        conv_zb<16, true>(a, smem, grid, s);
+        return;
     }
+    switch (NB) {
+        case 16: conv_zb<16>(a, smem, grid, s); break;
+        case 32: conv_zb<32>(a, smem, grid, s); break;
+        case 48: conv_zb<48>(a, smem, grid, s); break;
+        default: conv_zb<64>(a, smem, grid, s); break;
+    }
+}
+
+void conv_tc(cdi_unet* u, const CG& gl, const bf16* in, int cin, const bf16* w, int N, const float* bias, bf16* out,
+             bool relu, const bf16* up = nullptr, int cup = 0) {
+    conv_launch({gl, in, up, cin, cup, w, bias, out, nullptr, nullptr, nullptr, N, relu ? 1 : 0, 0, 0, 0, 0, u->tc_err},
+                false, u->stream);
+}
+
+// the first layer from the input pairs
+void conv_first(cdi_unet* u) {
+    conv_launch({u->g[0], u->xp, nullptr, 16, 0, u->Wk[0], u->B[0], u->e0, nullptr, nullptr, nullptr, 16, 1, 0, 0, 0, 0,
+                 u->tc_err}, true, u->stream);
+}
+
+// the last 3x3x3 layer with the head in its read-out (y only; d0 is not stored); in: [up (32 channels), in (16)]
+void conv_last(cdi_unet* u, const bf16* in, const bf16* up, float* y) {
+    conv_launch({u->g[0], in, up, 48, 32, u->Wk[6], u->B[6], nullptr, u->Wb[7], u->B[7], y, 16, 1, 0, 0, 0, 0,
+                 u->tc_err}, false, u->stream);
 }
 
 // y = conv(in) for layer l on level grid gl into out (stride, offset)
@@ -1306,14 +1441,15 @@ void refresh_weights(cdi_unet* u) {
     u->weights_ready = true;
 }
 
-// forward pass from u->x to u->y (FP32).  With keep_concat the decoder inputs
-// [up(coarser), skip] are stored (the weight gradients read them); otherwise the
-// tcgen05 convolution gathers them while staging its input tiles.
-void forward(cdi_unet* u, bool keep_concat = true) {
+// forward pass from the input (u->xp; u->x for the mma.sync kernels) to y (FP32).  With keep (training) every
+// activation the gradients read is stored: the decoder inputs [up(coarser), skip] and d0; otherwise the tcgen05
+// convolution gathers the former while staging its input tiles and only uses the latter for the head.
+void forward(cdi_unet* u, bool keep, float* y) {
     const CG* g = u->g;
     cudaStream_t s = u->stream;
-    const bool fuse = !keep_concat && u->use_tc;
-    conv_fwd<false>(u, 0, g[0], u->x, u->e0, 16, 0, true);
+    const bool fuse = !keep && u->use_tc;
+    if (u->use_tc) conv_first(u);
+    else conv_fwd<false>(u, 0, g[0], u->x, u->e0, 16, 0, true);
     k_pool<<<blocks(g[1].N * 2L), 256, 0, s>>>(g[0], u->e0, 16, u->p0);
     conv_fwd<false>(u, 1, g[1], u->p0, u->e1, 32, 0, true);
     k_pool<<<blocks(g[2].N * 4L), 256, 0, s>>>(g[1], u->e1, 32, u->p1);
@@ -1324,22 +1460,21 @@ void forward(cdi_unet* u, bool keep_concat = true) {
     if (fuse) {
         conv_tc(u, g[2], u->e2, 192, u->Wk[4], 64, u->B[4], u->d2, true, u->b, 128);
         conv_tc(u, g[1], u->e1, 96, u->Wk[5], 32, u->B[5], u->d1, true, u->d2, 64);
-        conv_tc(u, g[0], u->e0, 48, u->Wk[6], 16, u->B[6], u->d0, true, u->d1, 32);
+        conv_last(u, u->e0, u->d1, y);
         g_launches += 3;
-    } else {
-        k_up<<<blocks(g[2].N * 16L), 256, 0, s>>>(g[2], u->b, 128, u->c2, 192, 0);
-        k_copy_ch<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2].N, u->e2, 64, 0, u->c2, 192, 128, 64);
-        conv_fwd<false>(u, 4, g[2], u->c2, u->d2, 64, 0, true);
-        k_up<<<blocks(g[1].N * 8L), 256, 0, s>>>(g[1], u->d2, 64, u->c1, 96, 0);
-        k_copy_ch<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1].N, u->e1, 32, 0, u->c1, 96, 64, 32);
-        conv_fwd<false>(u, 5, g[1], u->c1, u->d1, 32, 0, true);
-        k_up<<<blocks(g[0].N * 4L), 256, 0, s>>>(g[0], u->d1, 32, u->c0, 48, 0);
-        k_copy_ch<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0].N, u->e0, 16, 0, u->c0, 48, 32, 16);
-        conv_fwd<false>(u, 6, g[0], u->c0, u->d0, 16, 0, true);
-        g_launches += 9;
+        return;
     }
-    conv_fwd<true>(u, 7, g[0], u->d0, u->y, 1, 0, false);
-    g_launches += 1;
+    k_up<<<blocks(g[2].N * 16L), 256, 0, s>>>(g[2], u->b, 128, u->c2, 192, 0);
+    k_copy_ch<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2].N, u->e2, 64, 0, u->c2, 192, 128, 64);
+    conv_fwd<false>(u, 4, g[2], u->c2, u->d2, 64, 0, true);
+    k_up<<<blocks(g[1].N * 8L), 256, 0, s>>>(g[1], u->d2, 64, u->c1, 96, 0);
+    k_copy_ch<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1].N, u->e1, 32, 0, u->c1, 96, 64, 32);
+    conv_fwd<false>(u, 5, g[1], u->c1, u->d1, 32, 0, true);
+    k_up<<<blocks(g[0].N * 4L), 256, 0, s>>>(g[0], u->d1, 32, u->c0, 48, 0);
+    k_copy_ch<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0].N, u->e0, 16, 0, u->c0, 48, 32, 16);
+    conv_fwd<false>(u, 6, g[0], u->c0, u->d0, 16, 0, true);
+    conv_fwd<true>(u, 7, g[0], u->d0, y, 1, 0, false);
+    g_launches += 10;
 }
 
 // gradients of the mean squared error (u->y against u->t) into gW, gB
@@ -1434,7 +1569,7 @@ cdi_status upload_x(cdi_unet* u, const double* x_host) {
     const long N = u->g[0].N;
     if (cudaMemcpyAsync(u->x2, x_host, (size_t)N * 2 * 8, cudaMemcpyHostToDevice, u->stream) != cudaSuccess)
         return ufail(u, CDI_ECUDA, "input upload failed");
-    k_input_host<<<blocks(N * 16), 256, 0, u->stream>>>((int)N, u->x2, u->x);
+    k_input_host<<<blocks(N), 256, 0, u->stream>>>((int)N, u->x2, u->xp, u->x);
     return CDI_OK;
 }
 
@@ -1451,10 +1586,10 @@ cudaError_t unet_predict_device(cdi_unet* u, const MG& mg, const T* phi_dev, dou
     const long N = u->g[0].N;
     const double rmax = fmax(rho1, rho2);
     k_solver_scales<<<1, 1, 0, s>>>(mg.scal + S_FNORM, (int)N, rmax * h * h, u->sd, u->sf);
-    k_input_solver<T><<<blocks(N * 16), 256, 0, s>>>((int)N, ops::fbuf<T>(mg.lv[0]), mg.scalf + SF_FMEAN_HI,
-                                                     phi_dev, (float)(rho1 - rho2), (float)rho2, (float)(1.0 / rmax),
-                                                     u->sd, u->sf, u->x);
-    forward(u, false);
+    k_input_solver<T><<<blocks(N), 256, 0, s>>>((int)N, ops::fbuf<T>(mg.lv[0]), mg.scalf + SF_FMEAN_HI, phi_dev,
+                                                (float)(rho1 - rho2), (float)rho2, (float)(1.0 / rmax), u->sd, u->sf,
+                                                u->xp, u->use_tc ? nullptr : u->x);
+    forward(u, false, u->y);
     k_output_solver<T><<<blocks(N), 256, 0, s>>>((int)N, u->y, u->sd, u->sf, ops::pbuf<T>(mg.lv[0]));
     g_launches += 3;
     u->stream = keep;
@@ -1576,7 +1711,7 @@ cdi_status cdi_unet_forward(cdi_unet* u, const double* x_host, double* y_host) {
     if (!u->weights_ready) refresh_weights(u);
     cdi_status st = upload_x(u, x_host);
     if (st) return st;
-    forward(u, false);
+    forward(u, false, u->y);
     const long N = u->g[0].N;
     std::vector<float> y(N);
     if (cudaMemcpyAsync(y.data(), u->y, (size_t)N * 4, cudaMemcpyDeviceToHost, u->stream) != cudaSuccess ||
@@ -1592,11 +1727,10 @@ cdi_status cdi_unet_forward_device(cdi_unet* u, const float* x_dev, float* y_dev
     if (!x_dev || !y_dev) return ufail(u, CDI_EINVAL, "null array");
     if (!u->weights_ready) refresh_weights(u);
     const long N = u->g[0].N;
-    k_input_dev<<<blocks(N * 16), 256, 0, u->stream>>>((int)N, x_dev, u->x);
-    forward(u, false);
+    if (u->use_tc) k_input_dev<<<blocks(N / 2), 256, 0, u->stream>>>((int)N, x_dev, u->xp);
+    else k_input_dev16<<<blocks(N), 256, 0, u->stream>>>((int)N, x_dev, u->xp, u->x);
+    forward(u, false, y_dev);
     g_launches += 1;
-    if (cudaMemcpyAsync(y_dev, u->y, (size_t)N * 4, cudaMemcpyDeviceToDevice, u->stream) != cudaSuccess)
-        return ufail(u, CDI_ECUDA, "output copy failed");
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return ufail(u, CDI_ECUDA, std::string("forward_device: ") + cudaGetErrorString(e));
     return CDI_OK;
@@ -1615,7 +1749,7 @@ cdi_status cdi_unet_train_step(cdi_unet* u, const double* x_host, const double* 
     if (st) return st;
     std::vector<float> t(t_host, t_host + N);
     cudaMemcpyAsync(u->t, t.data(), (size_t)N * 4, cudaMemcpyHostToDevice, u->stream);
-    forward(u);
+    forward(u, true, u->y);
     backward(u);
     float part = 0.f;
     cudaMemcpyAsync(&part, u->part, 4, cudaMemcpyDeviceToHost, u->stream);
