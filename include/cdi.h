@@ -283,11 +283,12 @@ void cdi_destroy(cdi_ctx* ctx);
  * Batched sweep: many independent problems (e.g. a theta_eq / slip length /
  * capillary number sweep) advanced together by ONE kernel launch.  Each
  * problem is an ordinary context (initialised, parameters set, workspace
- * bound, state set); the batch only schedules them: one CTA takes one
- * instance (largest first) and runs all its steps, so instances never wait
- * for each other.  The arithmetic of every instance is exactly that of
- * cdi_step (Sec. 4 time step), so results equal those of stepping each
- * context alone.  All instances need the same dimension and precision and
+ * bound, state set); the batch only schedules them: one CTA, or one cluster
+ * of 2 to 16 CTAs where the largest instances would outlast the rest, takes
+ * one instance (largest first) and runs all its steps, so instances never
+ * wait for each other.  The arithmetic of every instance is that of cdi_step
+ * (Sec. 4 time step), so results equal those of stepping each context alone
+ * up to the order of the sums over the grid.  All instances need the same dimension and precision and
  * must stay alive while the batch exists.
  * ------------------------------------------------------------------------- */
 typedef struct cdi_batch cdi_batch;

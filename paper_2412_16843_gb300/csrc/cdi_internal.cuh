@@ -352,6 +352,7 @@ void launch_contact_line(const Geom& g, int wall, const double* cols, MG& mg, cu
 // persistent step kernel (k_persist.cu)
 // ---------------------------------------------------------------------------
 constexpr int kPersistThreads = 512;
+constexpr int kMaxCluster = 16;  // CTAs of one cluster (above 8: non-portable)
 
 // per-instance outcome of one launch (zeroed before every launch)
 struct InstStats {
@@ -429,9 +430,10 @@ cudaError_t persist_prepare(int dim, size_t smem, int* grid);
 template <typename T>
 cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, cudaStream_t s);
 template <typename T>
-cudaError_t batch_prepare(int dim, int threads, size_t smem, int* grid);
+cudaError_t batch_prepare(int dim, int threads, size_t smem, int cluster, int* groups);  // groups: CTAs or clusters resident at once
 template <typename T>
-cudaError_t launch_batch_persist(BatchArgs<T>& B, int dim, int threads, size_t smem, int grid, cudaStream_t s);
+cudaError_t launch_batch_persist(BatchArgs<T>& B, int dim, int threads, size_t smem, int cluster, int groups,
+                                 cudaStream_t s);
 
 // number of kernel launches issued since the counter was reset (host side)
 extern thread_local long g_launches;

@@ -15,7 +15,12 @@
 //   size-sorted descriptor array) and runs all its steps alone, so every
 //   barrier is a __syncthreads and no CTA ever waits for another.
 //
-// Both run the same step code, written once against an executor X that
+// k_batch_cluster: the same with a thread-block cluster in the place of a CTA
+//   (barriers are hardware cluster barriers, reductions go through distributed
+//   shared memory), for batches whose largest instances would outlast the rest
+//   on one SM each.
+//
+// All run the same step code, written once against an executor X that
 // supplies the thread range, the barrier and the reductions.  In both, the
 // multigrid levels that fit in shared memory are solved by one CTA there.
 #include "ops.cuh"
@@ -155,6 +160,58 @@ struct BlockX {
     __device__ bool reduce(double v, double& out) {
         out = block_reduce_all<MAX>(v);
         return true;
+    }
+};
+
+// the CTAs of one thread-block cluster (hardware barrier; every CTA of a cluster is resident)
+struct ClusterX {
+    unsigned rank, size;
+    double* slots;  // this CTA's shared memory, [2][kMaxCluster]: the cluster's partials
+    int red;
+    using Ld = LG;
+    __device__ int tid() const { return (int)(rank * blockDim.x + threadIdx.x); }
+    __device__ int nth() const { return (int)(size * blockDim.x); }
+    __device__ int spread() const { return (int)(threadIdx.x * size + rank); }
+    __device__ bool tail_cta() const { return rank == 0; }
+    __device__ bool leader() const { return rank == 0 && threadIdx.x == 0; }
+    __device__ bool sync() {
+        cluster_barrier();
+        return true;
+    }
+    // each CTA writes its partial into every CTA's slots; two sets in turn, so a set is written again only after
+    // the barrier of the next reduction, which every reader of this one has passed
+    template <bool MAX>
+    __device__ bool reduce(double v, double& out) {
+        double* set = slots + (red++ & 1) * kMaxCluster;
+        v = block_reduce_all<MAX>(v);
+        if (threadIdx.x < size) st_cluster(set + rank, threadIdx.x, v);
+        cluster_barrier();
+        out = block_reduce_all<MAX>(threadIdx.x < size ? set[threadIdx.x] : 0.0);
+        return true;
+    }
+    __device__ static void cluster_barrier() {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    __device__ static unsigned remote(const void* p, unsigned r) {
+        unsigned a;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(r));
+        return a;
+    }
+    __device__ static void st_cluster(double* p, unsigned r, double v) {
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote(p, r)), "d"(v) : "memory");
+    }
+    __device__ static void st_cluster(int* p, unsigned r, int v) {
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(p, r)), "r"(v) : "memory");
+    }
+    __device__ static unsigned cluster_rank() {
+        unsigned r;
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+        return r;
+    }
+    __device__ static unsigned cluster_size() {
+        unsigned r;
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+        return r;
     }
 };
 
@@ -658,6 +715,32 @@ __global__ void __launch_bounds__(NT, 1) k_batch_persist(BatchArgs<T> B) {
     }
 }
 
+template <typename T, int DIM, int NT>
+__global__ void __launch_bounds__(NT, 1) k_batch_cluster(BatchArgs<T> B) {
+    extern __shared__ double smd[];
+    float* sm = reinterpret_cast<float*>(smd);
+    __shared__ int s_inst;
+    __shared__ double s_slots[2 * kMaxCluster];
+    __shared__ __align__(16) InstArgs<T> sA;
+    const unsigned rank = ClusterX::cluster_rank(), size = ClusterX::cluster_size();
+    for (;;) {
+        ClusterX::cluster_barrier();  // s_inst and sA of the previous instance are no longer read
+        if (rank == 0 && threadIdx.x == 0) {
+            const int i = atomicAdd(B.counter, 1);
+            for (unsigned r = 0; r < size; ++r) ClusterX::st_cluster(&s_inst, r, i);
+        }
+        ClusterX::cluster_barrier();
+        const int i = s_inst;
+        if (i >= B.n_inst) return;
+        const int4* src = reinterpret_cast<const int4*>(B.insts + i);
+        int4* dst = reinterpret_cast<int4*>(&sA);
+        for (int w = threadIdx.x; w < (int)(sizeof(InstArgs<T>) / sizeof(int4)); w += blockDim.x) dst[w] = src[w];
+        __syncthreads();
+        ClusterX x{rank, size, s_slots, 0};
+        run_steps<T, DIM>(sA, x, B.nsteps, B.stats + i, sm);
+    }
+}
+
 }  // namespace
 
 // shared-memory layout of the FP32 tail levels and the FP64 dense-solve scratch; returns bytes
@@ -729,45 +812,77 @@ cudaError_t persist_prepare(int dim, size_t smem, int* grid) {
 }
 
 template <typename T, int NT>
-static const void* batch_fn(int dim) {
+static const void* batch_fn(int dim, bool cluster) {
+    if (cluster) return (dim == 2) ? (const void*)k_batch_cluster<T, 2, NT> : (const void*)k_batch_cluster<T, 3, NT>;
     return (dim == 2) ? (const void*)k_batch_persist<T, 2, NT> : (const void*)k_batch_persist<T, 3, NT>;
 }
 template <typename T>
-static const void* batch_fn_threads(int dim, int threads) {
+static const void* batch_fn_threads(int dim, int threads, bool cluster) {
     switch (threads) {
-        case 256: return batch_fn<T, 256>(dim);
-        case 1024: return batch_fn<T, 1024>(dim);
-        default: return batch_fn<T, 512>(dim);
+        case 256: return batch_fn<T, 256>(dim, cluster);
+        case 1024: return batch_fn<T, 1024>(dim, cluster);
+        default: return batch_fn<T, 512>(dim, cluster);
     }
 }
 
 template <typename T>
-cudaError_t batch_prepare(int dim, int threads, size_t smem, int* grid) {
-    const void* fn = batch_fn_threads<T>(dim, threads);
+cudaError_t batch_prepare(int dim, int threads, size_t smem, int cluster, int* groups) {
+    const void* fn = batch_fn_threads<T>(dim, threads, cluster > 1);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (cluster > 1) {
+        if (cluster > 8 && (e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
+                               cudaSuccess)
+            return e;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cfg.gridDim = dim3(nsm / cluster * cluster);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim = {(unsigned)cluster, 1, 1};
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if ((e = cudaOccupancyMaxActiveClusters(&per, fn, &cfg)) != cudaSuccess) return e;
+        if (per < 1) return cudaErrorInvalidConfiguration;
+        *groups = per;
+        return cudaSuccess;
+    }
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem)) != cudaSuccess) return e;
     if (per < 1) return cudaErrorInvalidConfiguration;
-    *grid = nsm * per;
+    *groups = nsm * per;
     return cudaSuccess;
 }
 
 template <typename T>
-cudaError_t launch_batch_persist(BatchArgs<T>& B, int dim, int threads, size_t smem, int grid, cudaStream_t s) {
+cudaError_t launch_batch_persist(BatchArgs<T>& B, int dim, int threads, size_t smem, int cluster, int groups,
+                                 cudaStream_t s) {
     void* args[] = {&B};
-    return cudaLaunchKernel(batch_fn_threads<T>(dim, threads), dim3(grid), dim3(threads), args, smem, s);
+    const void* fn = batch_fn_threads<T>(dim, threads, cluster > 1);
+    if (cluster == 1) return cudaLaunchKernel(fn, dim3(groups), dim3(threads), args, smem, s);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cfg.gridDim = dim3((unsigned)(groups * cluster));
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)cluster, 1, 1};
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 template cudaError_t launch_step_persist<double>(PersistArgs<double>&, size_t, int, cudaStream_t);
 template cudaError_t launch_step_persist<float>(PersistArgs<float>&, size_t, int, cudaStream_t);
 template cudaError_t persist_prepare<double>(int, size_t, int*);
 template cudaError_t persist_prepare<float>(int, size_t, int*);
-template cudaError_t batch_prepare<double>(int, int, size_t, int*);
-template cudaError_t batch_prepare<float>(int, int, size_t, int*);
-template cudaError_t launch_batch_persist<double>(BatchArgs<double>&, int, int, size_t, int, cudaStream_t);
-template cudaError_t launch_batch_persist<float>(BatchArgs<float>&, int, int, size_t, int, cudaStream_t);
+template cudaError_t batch_prepare<double>(int, int, size_t, int, int*);
+template cudaError_t batch_prepare<float>(int, int, size_t, int, int*);
+template cudaError_t launch_batch_persist<double>(BatchArgs<double>&, int, int, size_t, int, int, cudaStream_t);
+template cudaError_t launch_batch_persist<float>(BatchArgs<float>&, int, int, size_t, int, int, cudaStream_t);
 
 }  // namespace cdi
