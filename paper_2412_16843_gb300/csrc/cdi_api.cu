@@ -836,6 +836,8 @@ void fill_inst(const cdi_ctx* c, InstArgs<T>& A, int lt, const PersistLayout& la
     A.npost = c->npost;
     A.gamma_param = c->gamma;
     A.dt = dt;
+    A.inv_cdt[0] = 1.0 / (0.5 * dt);
+    A.inv_cdt[1] = 1.0 / dt;
     for (int k = 0; k < 4; ++k)
         for (int j = 0; j < 2; ++j) A.hist[k][j] = c->hist[k][j];
     A.hist_step0 = c->hist_steps;
@@ -846,7 +848,7 @@ void fill_inst(const cdi_ctx* c, InstArgs<T>& A, int lt, const PersistLayout& la
 // and stage buffers once per finished step
 cdi_status apply_stats(cdi_ctx* c, const InstStats& h, const char* who) {
     c->last_cycles = h.last_cycles;
-    c->last_resid = h.last_resid;
+    c->last_resid = h.last_fsq == 0.0 ? 0.0 : std::sqrt(h.last_rsq) / std::sqrt(h.last_fsq);
     c->max_cycles_step = h.max_cycles;
     c->total_cycles_call = h.total_cycles;
     c->hist_steps += h.steps_done;
@@ -858,7 +860,7 @@ cdi_status apply_stats(cdi_ctx* c, const InstStats& h, const char* who) {
     char b[240];
     if (h.status == CDI_ENOCONV)
         snprintf(b, sizeof b, "%spressure solve: %d V-cycles left relative residual %.3e > tol %.3e (step %d)", who,
-                 h.last_cycles, h.last_resid, c->tol, h.steps_done);
+                 h.last_cycles, c->last_resid, c->tol, h.steps_done);
     else if (h.status == CDI_ETIMEOUT)
         snprintf(b, sizeof b, "%sa grid barrier of the persistent step kernel timed out (step %d)", who, h.steps_done);
     else

@@ -53,6 +53,7 @@ struct Geom {
     double ih, ih2;         // 1/h, 1/h^2
     float hf, ihf, ih2f;    // FP32 copies (1/h and 1/h^2 rounded from the FP32 h and h^2)
     FastDiv fd0, fd1;  // division by n[0] and by n[1]
+    FastDiv fdh;       // division by n[0] / 2 (cells of one colour in a row)
 };
 
 // 1/h and 1/h^2 in the arithmetic type of a kernel.  On GB300 an FP64
@@ -80,6 +81,7 @@ inline Geom make_geom(int D, const int n[3], double h) {
     g.ih2f = 1.f / (float)(h * h);
     g.fd0.init((unsigned)n[0]);
     g.fd1.init((unsigned)n[1]);
+    g.fdh.init(n[0] > 1 ? (unsigned)n[0] / 2 : 1u);
     return g;
 }
 
@@ -189,6 +191,20 @@ __host__ __device__ __forceinline__ IJK shift(const Geom& g, IJK q, int a, int s
     return q;
 }
 __host__ __device__ __forceinline__ long idx(const Geom& g, const IJK& q) { return encode(g, q.i, q.j, q.k); }
+
+// index of the low / high neighbour of cell c = idx(g, q) along axis a
+// (periodic axes wrap; not past a wall): idx(g, shift(g, q, a, -1 / 1))
+// without encoding the neighbour's coordinates
+__host__ __device__ __forceinline__ long lo_idx(const Geom& g, const IJK& q, long c, int a) {
+    if (a == g.W) return c - g.NP;
+    const int st = a == 0 ? 1 : g.n[0];
+    return coord(q, a) == 0 ? c + (long)(st * (g.n[a] - 1)) : c - st;
+}
+__host__ __device__ __forceinline__ long hi_idx(const Geom& g, const IJK& q, long c, int a) {
+    if (a == g.W) return c + g.NP;
+    const int st = a == 0 ? 1 : g.n[0];
+    return coord(q, a) == g.n[a] - 1 ? c - (long)(st * (g.n[a] - 1)) : c + st;
+}
 
 template <typename T>
 __host__ __device__ __forceinline__ T clampv(T x, T lo, T hi) { return x < lo ? lo : (x > hi ? hi : x); }
@@ -362,7 +378,7 @@ struct InstStats {
     int total_cycles;  // V-cycles of all solves in this launch
     int steps_done;
     int pad;
-    double last_resid;
+    double last_rsq, last_fsq;  // squared norms of the last solve's residual and right-hand side
 };
 
 // control block of the single-grid persistent kernel in the workspace
@@ -396,6 +412,7 @@ struct __align__(16) InstArgs : PersistLayout {
     double tol;
     int max_vcycles, warm, npre, npost;
     double gamma_param, dt;
+    double inv_cdt[2];   // 1 / (c dt) of the projections of stages 0, 1 (c = 1/2) and 2, 3 (c = 1)
     // first guess by extrapolation in time (CDI_WARM_EXTRAP): the pressure of
     // RK stage k of the last two steps, hist[k][s & 1] written at step s
     double* hist[4][2];

@@ -672,8 +672,8 @@ template <int DIM>
 __global__ void k_coarse(Geom g, const float* b0, const float* b1, const float* b2, const float* ainv,
                          const float* r, float* e) {
     const float* beta[3] = {b0, b1, b2};
-    __shared__ double rd[kMaxCoarse], ed[kMaxCoarse], rr[kMaxCoarse];
-    ops::coarse_apply_block<Ld, float, DIM>(g, beta, ainv, r, e, rd, ed, rr);
+    __shared__ double ed[kMaxCoarse];
+    ops::coarse_apply_block<Ld, float, DIM>(g, beta, ainv, r, e, ed);
 }
 
 template <typename T>

@@ -43,22 +43,34 @@ __device__ __forceinline__ double warp_max(double v) {
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
     return v;
 }
-// block-wide sum or max, returned to every thread of the block
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
+__device__ __forceinline__ bool finite(double v) {
+    return ((__double_as_longlong(v) >> 52) & 0x7ff) != 0x7ff;
+}
+// Block-wide sum or max in thread 0 (every thread calls).  An FP64 instruction
+// of a warp occupies its scheduler's pipe for tens of cycles, so warps whose
+// values are all zero (no cells of a small grid) skip their tree.
 template <bool MAX>
-__device__ double block_reduce_all(double v) {
+__device__ double block_reduce(double v) {
     __shared__ double sh[32];
-    __shared__ double res;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    v = MAX ? warp_max(v) : warp_sum(v);
+    if (__any_sync(0xffffffffu, nonzero(v))) v = MAX ? warp_max(v) : warp_sum(v);
     __syncthreads();
     if (lane == 0) sh[wid] = v;
     __syncthreads();
     if (wid == 0) {
         const int nw = (blockDim.x + 31) >> 5;
-        double x = lane < nw ? sh[lane] : 0.0;
-        x = MAX ? warp_max(x) : warp_sum(x);
-        if (lane == 0) res = x;
+        v = lane < nw ? sh[lane] : 0.0;
+        if (__any_sync(0xffffffffu, nonzero(v))) v = MAX ? warp_max(v) : warp_sum(v);
     }
+    return v;
+}
+// what a reduction returns to every thread: its value, or its value over n
+// (one warp divides: the division is about ten FP64 instructions)
+template <bool MAX>
+__device__ double bcast_result(double v, double n) {
+    __shared__ double res;
+    if (threadIdx.x == 0) res = n == 1.0 ? v : v / n;
     __syncthreads();
     return res;
 }
@@ -90,7 +102,10 @@ struct GridX {
     int red;
     unsigned long long epoch;  // barriers passed by this CTA
     using Ld = LG;
-    __device__ int tid() const { return blockIdx.x * blockDim.x + threadIdx.x; }
+    // consecutive groups of 32 cells go to consecutive CTAs: a grid of fewer cells than threads is spread over all
+    // SMs instead of filling the first few (their FP64 pipes bind the stage phases: the cell phase of a 64 x 32 grid
+    // took 33k cycles on four SMs)
+    __device__ int tid() const { return ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31); }
     __device__ int nth() const { return gridDim.x * blockDim.x; }
     // the thread's first index of a loop with stride nth() whose consecutive
     // indices go to consecutive CTAs
@@ -131,16 +146,26 @@ struct GridX {
         __syncthreads();
         return ok != 0;
     }
+    // the CTAs' partials are added by one warp of every CTA in the same order; out: the sum (or maximum) over n
     template <bool MAX>
-    __device__ bool reduce(double v, double& out) {
+    __device__ bool reduce(double v, double& out, double n = 1.0) {
         double* part = partials + (red++ & 1) * kPartials;
-        v = block_reduce_all<MAX>(v);
+        v = block_reduce<MAX>(v);
         if (threadIdx.x == 0) part[blockIdx.x] = v;
         if (!sync()) return false;
-        double s = 0.0;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-            s = MAX ? fmax(s, __ldcg(part + b)) : s + __ldcg(part + b);
-        out = block_reduce_all<MAX>(s);
+        if (threadIdx.x < 32) {
+            constexpr int U = 5;  // loads in flight before the first sum (152 CTAs: all)
+            double s = 0.0;
+            for (int b0 = threadIdx.x; b0 < (int)gridDim.x; b0 += 32 * U) {
+                double t[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) t[u] = b0 + 32 * u < (int)gridDim.x ? __ldcg(part + b0 + 32 * u) : 0.0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) s = MAX ? fmax(s, t[u]) : s + t[u];
+            }
+            v = MAX ? warp_max(s) : warp_sum(s);
+        }
+        out = bcast_result<MAX>(v, n);
         return true;
     }
 };
@@ -157,8 +182,8 @@ struct BlockX {
         return true;
     }
     template <bool MAX>
-    __device__ bool reduce(double v, double& out) {
-        out = block_reduce_all<MAX>(v);
+    __device__ bool reduce(double v, double& out, double n = 1.0) {
+        out = bcast_result<MAX>(block_reduce<MAX>(v), n);
         return true;
     }
 };
@@ -169,7 +194,7 @@ struct ClusterX {
     double* slots;  // this CTA's shared memory, [2][kMaxCluster]: the cluster's partials
     int red;
     using Ld = LG;
-    __device__ int tid() const { return (int)(rank * blockDim.x + threadIdx.x); }
+    __device__ int tid() const { return (int)(((threadIdx.x >> 5) * size + rank) * 32 + (threadIdx.x & 31)); }
     __device__ int nth() const { return (int)(size * blockDim.x); }
     __device__ int spread() const { return (int)(threadIdx.x * size + rank); }
     __device__ bool tail_cta() const { return rank == 0; }
@@ -181,12 +206,19 @@ struct ClusterX {
     // each CTA writes its partial into every CTA's slots; two sets in turn, so a set is written again only after
     // the barrier of the next reduction, which every reader of this one has passed
     template <bool MAX>
-    __device__ bool reduce(double v, double& out) {
+    __device__ bool reduce(double v, double& out, double n = 1.0) {
         double* set = slots + (red++ & 1) * kMaxCluster;
-        v = block_reduce_all<MAX>(v);
-        if (threadIdx.x < size) st_cluster(set + rank, threadIdx.x, v);
+        v = block_reduce<MAX>(v);
+        if (threadIdx.x < 32) {
+            v = __shfl_sync(0xffffffffu, v, 0);
+            if (threadIdx.x < size) st_cluster(set + rank, threadIdx.x, v);
+        }
         cluster_barrier();
-        out = block_reduce_all<MAX>(threadIdx.x < size ? set[threadIdx.x] : 0.0);
+        if (threadIdx.x < 32) {
+            v = threadIdx.x < size ? set[threadIdx.x] : 0.0;
+            v = MAX ? warp_max(v) : warp_sum(v);
+        }
+        out = bcast_result<MAX>(v, n);
         return true;
     }
     __device__ static void cluster_barrier() {
@@ -246,8 +278,9 @@ __device__ __forceinline__ void tail_pass(const SmLevel& L, const float* const* 
     ops::colour_pass(
         t0, half, nt,
         [&](int k, long& c) {
-            c = ops::colour_cell(L.g, col, k);
-            return ops::rbgs_val<LP, float, DIM>(L.g, bl, L.e, L.r, c);
+            IJK q;
+            c = ops::colour_cell(L.g, col, k, q);
+            return ops::rbgs_val<LP, float, DIM>(L.g, bl, L.e, L.r, q, c);
         },
         [&](long c, float v) { L.e[c] = v; });
 }
@@ -339,9 +372,7 @@ __device__ void tail_vcycle(const InstArgs<T>& A, bool first, float* sm) {
             __shared__ float shv;
             ops::coarse_invert_block<LP, float, DIM>(C.g, bc, Asm, reinterpret_cast<float*>(sd + A.sm_fct), &shv);
         }
-        double* cs = sd + A.sm_bb;  // FP64 scratch of the solve: 3 x kMaxCoarse doubles (sm_bb, then sm_fct)
-        ops::coarse_apply_block<LP, float, DIM>(C.g, bc, A.ainv ? A.ainv : Asm, C.r, C.e, cs, cs + kMaxCoarse,
-                                                sd + A.sm_fct);
+        ops::coarse_apply_block<LP, float, DIM>(C.g, bc, A.ainv ? A.ainv : Asm, C.r, C.e, sd + A.sm_bb);
     }
     // up: in shared memory a separate prolongation pass is cheaper than
     // prolonging the neighbours of every red cell on the fly
@@ -387,9 +418,10 @@ __device__ bool vcycle(const InstArgs<T>& A, X& x, bool first, float* sm) {
                 ops::colour_pass(
                     tid, half, nth,
                     [&](int k, long& c) {
-                        c = ops::colour_cell(L.g, col, k);
-                        return l == 0 ? ops::rbgs_rho_val<L_, DIM>(L.g, L.rho0, L.e, L.r, c)
-                                      : ops::rbgs_val<L_, float, DIM>(L.g, bl, L.e, L.r, c);
+                        IJK q;
+                        c = ops::colour_cell(L.g, col, k, q);
+                        return l == 0 ? ops::rbgs_rho_val<L_, DIM>(L.g, L.rho0, L.e, L.r, q, c)
+                                      : ops::rbgs_val<L_, float, DIM>(L.g, bl, L.e, L.r, q, c);
                     },
                     [&](long c, float v) { L.e[c] = v; });
                 if (!x.sync()) return false;
@@ -420,14 +452,15 @@ __device__ bool vcycle(const InstArgs<T>& A, X& x, bool first, float* sm) {
                 ops::colour_pass(
                     tid, half, nth,
                     [&](int k, long& c) {
-                        c = ops::colour_cell(L.g, col, k);
+                        IJK q;
+                        c = ops::colour_cell(L.g, col, k, q);
                         if (pro)
-                            return l == 0 ? ops::rbgs_rho_val<L_, DIM, ops::kNbProlong>(L.g, L.rho0, L.e, L.r, c,
+                            return l == 0 ? ops::rbgs_rho_val<L_, DIM, ops::kNbProlong>(L.g, L.rho0, L.e, L.r, q, c,
                                                                                       &C.g, C.e)
-                                          : ops::rbgs_val<L_, float, DIM, ops::kNbProlong>(L.g, bl, L.e, L.r, c,
+                                          : ops::rbgs_val<L_, float, DIM, ops::kNbProlong>(L.g, bl, L.e, L.r, q, c,
                                                                                          &C.g, C.e);
-                        return l == 0 ? ops::rbgs_rho_val<L_, DIM>(L.g, L.rho0, L.e, L.r, c)
-                                      : ops::rbgs_val<L_, float, DIM>(L.g, bl, L.e, L.r, c);
+                        return l == 0 ? ops::rbgs_rho_val<L_, DIM>(L.g, L.rho0, L.e, L.r, q, c)
+                                      : ops::rbgs_val<L_, float, DIM>(L.g, bl, L.e, L.r, q, c);
                     },
                     [&](long c, float v) {
                         L.e[c] = v;
@@ -435,7 +468,8 @@ __device__ bool vcycle(const InstArgs<T>& A, X& x, bool first, float* sm) {
                     });
                 if (last) {  // the other colour is final already
                     for (int k = tid; k < half; k += nth) {
-                        const long c = ops::colour_cell(L.g, 0, k);
+                        IJK q;
+                        const long c = ops::colour_cell(L.g, 0, k, q);
                         P0[c] = ops::p_add(L_::ld(P0 + c), L_::ld(L.e + c));
                     }
                     updated = true;
@@ -489,7 +523,7 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
     const MGLevel L0 = A.lv[0];
     PT<T>* P0 = ops::pbuf<T>(L0);
     FT<T>* F0 = ops::fbuf<T>(L0);
-    const T ih = g_ih<T>(g), inv_cdt = (T)(1.0 / cdt);
+    const T ih = g_ih<T>(g), inv_cdt = (T)(stage < 2 ? A.inv_cdt[0] : A.inv_cdt[1]);  // 1 / cdt
     const T* uc[3] = {u[0], u[1], u[2]};
     ops::SumAcc<T> s;
     for (int c = tid; c < (int)g.N; c += nth) {
@@ -497,9 +531,8 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
         F0[c] = v;
         s.add(v);
     }
-    double sum;
-    if (!x.template reduce<false>(s.value(), sum)) return false;
-    const double mean = sum / (double)g.N;
+    double mean;
+    if (!x.template reduce<false>(s.value(), mean, (double)g.N)) return false;
     // FP64 form: f is centred in place; FP32-mixed form: the residual removes the mean
     const float2 fmean = ops::dfl::from_double(mean);
     T s2 = T(0);
@@ -524,7 +557,11 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
         ops::coef0_at<L_, T, DIM>(g, A.ph, phi, L0.beta, L0.bf, L0.rho0, t);
     double fsq;
     if (!x.template reduce<false>((double)s2, fsq)) return false;
-    const double fn = sqrt(fsq);
+    // ||r|| > tol ||f|| is tested on the squares (an FP64 square root in every warp and V-cycle cost 3k cycles), and on
+    // the norms only where tol^2 ||f||^2 could underflow
+    const double lim = A.tol * A.tol * fsq;
+    const bool squares = fsq > 1e-200;
+    auto above = [&](double rsq) { return squares ? rsq > lim : sqrt(rsq) > A.tol * sqrt(fsq); };
     for (int l = 1; l < A.lt; ++l) {
         const MGLevel F = A.lv[l - 1];
         const MGLevel C = A.lv[l];
@@ -535,14 +572,13 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
     }
     double rsq;
     if (!x.template reduce<false>(resid_local<L_, T, DIM>(L0, fmean, tid, nth), rsq)) return false;
-    double rn = sqrt(rsq);
-    if (!isfinite(fn) || !isfinite(rn)) {
+    if (!finite(fsq) || !finite(rsq)) {
         set_status(x, S, CDI_ENAN);
         return false;
     }
     int cyc = 0;
     PT<T>* hput = extrap ? reinterpret_cast<PT<T>*>(A.hist[stage][sg & 1]) : nullptr;
-    if (fn == 0.0) {
+    if (!nonzero(fsq)) {
         for (int c = tid; c < (int)g.N; c += nth) {
             P0[c] = ops::p_zero<T>();
             if (extrap) hput[c] = ops::p_zero<T>();
@@ -550,22 +586,22 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
         if (!x.sync()) return false;
     } else {
         bool first = true;
-        while (rn > A.tol * fn && cyc < A.max_vcycles) {
+        while (cyc < A.max_vcycles && above(rsq)) {
             if (!vcycle<T, DIM>(A, x, first, sm)) return false;
             first = false;
             if (!x.template reduce<false>(resid_local<L_, T, DIM>(L0, fmean, tid, nth), rsq)) return false;
-            rn = sqrt(rsq);
             ++cyc;
-            if (!isfinite(rn)) {
+            if (!finite(rsq)) {
                 set_status(x, S, CDI_ENAN);
                 return false;
             }
         }
-        if (rn > A.tol * fn) {
+        if (cyc >= A.max_vcycles && above(rsq)) {
             set_status(x, S, CDI_ENOCONV);
             if (x.leader()) {
                 S->last_cycles = cyc;
-                S->last_resid = rn / fn;
+                S->last_rsq = rsq;
+                S->last_fsq = fsq;
             }
             return false;
         }
@@ -578,9 +614,8 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
             for (int c = tid; c < (int)g.N; c += nth) a = ops::dfl::add(a, L_::ld(P0 + c));
             ps = ops::dfl::to_double(a);
         }
-        double psum;
-        if (!x.template reduce<false>(ps, psum)) return false;
-        const double pmean = psum / (double)g.N;
+        double pmean;
+        if (!x.template reduce<false>(ps, pmean, (double)g.N)) return false;
         const float2 pm2 = ops::dfl::from_double(pmean);
         for (int c = tid; c < (int)g.N; c += nth) {
             const PT<T> v = ops::p_sub(L_::ld(P0 + c), pmean, pm2);
@@ -591,7 +626,8 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
     }
     if (x.leader()) {
         S->last_cycles = cyc;
-        S->last_resid = fn == 0.0 ? 0.0 : rn / fn;
+        S->last_rsq = rsq;
+        S->last_fsq = fsq;
         S->total_cycles += cyc;
         if (cyc > S->max_cycles) S->max_cycles = cyc;
     }

@@ -61,7 +61,7 @@ __device__ __forceinline__ void d12(const Geom& g, const T* s, const IJK& q, lon
         d2 = (sp - T(2) * s0 + sm) * ih2;
         return;
     }
-    T sm = L::ld(s + idx(g, shift(g, q, b, -1))), s0 = L::ld(s + c), sp = L::ld(s + idx(g, shift(g, q, b, 1)));
+    T sm = L::ld(s + lo_idx(g, q, c, b)), s0 = L::ld(s + c), sp = L::ld(s + hi_idx(g, q, c, b));
     d1 = (sp - sm) * half_ih;
     d2 = (sp - T(2) * s0 + sm) * ih2;
 }
@@ -357,11 +357,11 @@ __device__ __forceinline__ void phi_rhs_at(const Geom& g, const PhysDev& ph, con
         T Flo = T(0), Fhi = T(0);
         const T ulo = L::ld(ua + c);
         if (!(a == W && r == 0)) {
-            long cL = idx(g, shift(g, q, a, -1));
+            long cL = lo_idx(g, q, c, a);
             Flo = phi_flux<L>(f.phi, na, cL, c, ulo, gamma, eps, ih, delta);
         }
         if (!(a == W && r == g.n[W] - 1)) {
-            long cR = idx(g, shift(g, q, a, 1));
+            long cR = hi_idx(g, q, c, a);
             long fi = (a == W) ? c + g.NP : cR;
             Fhi = phi_flux<L>(f.phi, na, c, cR, L::ld(ua + fi), gamma, eps, ih, delta);
         }
@@ -388,12 +388,12 @@ __device__ void mom_at(const Geom& g, const PhysDev& ph, const StageFields<T>& f
         const T* ua = f.u[a];
         if (a == W && coord(q, W) == 0) { f.rm[a][c] = T(0); continue; }  // wall face
         const long cR = c;
-        const long cL = idx(g, shift(g, q, a, -1));
+        const long cL = lo_idx(g, q, c, a);
         T adv = T(0), vis = T(0);
 #pragma unroll
         for (int b = 0; b < DIM; ++b) {
             if (b == a) {
-                const long fRlo = c, fRhi = (a == W) ? c + g.NP : idx(g, shift(g, q, a, 1));
+                const long fRlo = c, fRhi = (a == W) ? c + g.NP : hi_idx(g, q, c, a);
                 const long fLlo = cL, fLhi = c;
                 const T* ma = f.m[a];
                 const T uRlo = L::ld(ua + fRlo), uRhi = L::ld(ua + fRhi), uLlo = L::ld(ua + fLlo);
@@ -464,7 +464,7 @@ __device__ __forceinline__ void stage_mom_at(const Geom& g, const PhysDev& ph, T
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         if (a == W && coord(q, W) == 0) { uk[a][c] = T(0); acc[a][c] = T(0); continue; }
-        const long cL = idx(g, shift(g, q, a, -1));
+        const long cL = lo_idx(g, q, c, a);
         const T rf0 = T(0.5) * ((drho * L::ld(phi0 + cL) + rho2) + (drho * L::ld(phi0 + c) + rho2));
         const T M0 = rf0 * L::ld(u0[a] + c);
         const T k = L::ld(rm[a] + c);
@@ -493,7 +493,7 @@ __device__ __forceinline__ T div_at(const Geom& g, const T* const* us, T ih, T i
     T div = T(0);
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        const long hi = (a == DIM - 1) ? c + g.NP : idx(g, shift(g, q, a, 1));
+        const long hi = (a == DIM - 1) ? c + g.NP : hi_idx(g, q, c, a);
         div += L::ld(us[a] + hi) - L::ld(us[a] + c);
     }
     return div * ih * inv_cdt;
@@ -521,7 +521,7 @@ __device__ __forceinline__ void coef0_at(const Geom& g, const PhysDev& ph, const
             bsf[a][t] = 0.f;
             continue;
         }
-        const long cL = idx(g, shift(g, q, a, -1));
+        const long cL = lo_idx(g, q, t, a);
         const T rf = T(0.5) * ((dr * L::ld(phi + cL) + rho2) + (dr * L::ld(phi + t) + rho2));
         const T b = T(1) / rf;
         if (f64) bs[a][t] = (double)b;
@@ -576,8 +576,8 @@ __device__ __forceinline__ void stencil_L(const Geom& g, const M* const* beta, c
             lo = wlo ? c : c - g.NP;
             hi = whi ? c : c + g.NP;
         } else {
-            lo = idx(g, shift(g, q, a, -1));
-            hi = idx(g, shift(g, q, a, 1));
+            lo = lo_idx(g, q, c, a);
+            hi = hi_idx(g, q, c, a);
         }
         const long fhi = (a == DIM - 1) ? c + g.NP : hi;
         const M bm = L::ld(beta[a] + c);
@@ -619,8 +619,8 @@ __device__ __forceinline__ void stencil_L_rho(const Geom& g, const float* rho, c
             lo = wlo ? c : c - g.NP;
             hi = whi ? c : c + g.NP;
         } else {
-            lo = idx(g, shift(g, q, a, -1));
-            hi = idx(g, shift(g, q, a, 1));
+            lo = lo_idx(g, q, c, a);
+            hi = hi_idx(g, q, c, a);
         }
         const float bm = (wlo ? 0.f : 1.f) * __fdividef(2.f, rc + L::ld(rho + lo));
         const float bp = (whi ? 0.f : 1.f) * __fdividef(2.f, rc + L::ld(rho + hi));
@@ -639,13 +639,16 @@ __device__ __forceinline__ float apply_L_rho(const Geom& g, const float* rho, co
 }
 
 // k-th cell of one colour ((i+j+k) even or odd); every extent of a smoothed level is even
-__device__ __forceinline__ long colour_cell(const Geom& g, int colour, long k) {
+__device__ __forceinline__ long colour_cell(const Geom& g, int colour, long k, IJK& q) {
     const unsigned half = (unsigned)g.n[0] >> 1;
-    const unsigned line = (unsigned)k / half;
+    const unsigned line = g.fdh.div((unsigned)k);
     const unsigned m = (unsigned)k - line * half;
-    const unsigned kk = g.fd1.div(line);
+    const unsigned kk = g.D == 3 ? g.fd1.div(line) : 0u;
     const unsigned j = line - kk * (unsigned)g.n[1];
     const unsigned i = 2u * m + ((colour + j + kk) & 1u);
+    q.i = (int)i;
+    q.j = (int)j;
+    q.k = (int)kk;
     return (long)(i + (unsigned)g.n[0] * line);
 }
 
@@ -682,9 +685,8 @@ __device__ __forceinline__ M prolong_val(const Geom& gf, const Geom& gc, const M
 
 // the new value of cell c (rbgs_at without the store)
 template <class L, typename M, int DIM, int NB = kNbStored>
-__device__ __forceinline__ M rbgs_val(const Geom& g, const M* const* beta, const M* p, const M* f, long c,
+__device__ __forceinline__ M rbgs_val(const Geom& g, const M* const* beta, const M* p, const M* f, const IJK& q, long c,
                                       const Geom* gc = nullptr, const M* pc = nullptr) {
-    const IJK q = decode(g, c);
     const M ih2 = g_ih2<M>(g);
     M diag, off;
     stencil_L<L, M, DIM>(
@@ -701,14 +703,14 @@ __device__ __forceinline__ M rbgs_val(const Geom& g, const M* const* beta, const
 template <class L, typename M, int DIM, int NB = kNbStored>
 __device__ __forceinline__ void rbgs_at(const Geom& g, const M* const* beta, M* p, const M* f, long c,
                                         const Geom* gc = nullptr, const M* pc = nullptr) {
-    p[c] = rbgs_val<L, M, DIM, NB>(g, beta, p, f, c, gc, pc);
+    p[c] = rbgs_val<L, M, DIM, NB>(g, beta, p, f, decode(g, c), c, gc, pc);
 }
 
 // level-0 smoothing value with density-formed coefficients (stencil_L_rho)
 template <class L, int DIM, int NB = kNbStored>
-__device__ __forceinline__ float rbgs_rho_val(const Geom& g, const float* rho, const float* p, const float* f, long c,
-                                              const Geom* gc = nullptr, const float* pc = nullptr) {
-    const IJK q = decode(g, c);
+__device__ __forceinline__ float rbgs_rho_val(const Geom& g, const float* rho, const float* p, const float* f,
+                                              const IJK& q, long c, const Geom* gc = nullptr,
+                                              const float* pc = nullptr) {
     float diag, off;
     stencil_L_rho<L, DIM>(
         g, rho, q, c, g.ih2f,
@@ -724,7 +726,7 @@ __device__ __forceinline__ float rbgs_rho_val(const Geom& g, const float* rho, c
 template <class L, int DIM, int NB = kNbStored>
 __device__ __forceinline__ void rbgs_rho_at(const Geom& g, const float* rho, float* p, const float* f, long c,
                                             const Geom* gc = nullptr, const float* pc = nullptr) {
-    p[c] = rbgs_rho_val<L, DIM, NB>(g, rho, p, f, c, gc, pc);
+    p[c] = rbgs_rho_val<L, DIM, NB>(g, rho, p, f, decode(g, c), c, gc, pc);
 }
 
 // One colour of a red-black pass over the cells k0, k0 + stride, ... < half
@@ -871,8 +873,8 @@ __device__ __forceinline__ float resid_df_at(const Geom& g, const float* const* 
             lo = r > 0 ? c - g.NP : c;
             hi = r < g.n[a] - 1 ? c + g.NP : c;
         } else {
-            lo = idx(g, shift(g, q, a, -1));
-            hi = idx(g, shift(g, q, a, 1));
+            lo = lo_idx(g, q, c, a);
+            hi = hi_idx(g, q, c, a);
         }
         const long fhi = (a == DIM - 1) ? c + g.NP : hi;
         const float bm = L::ld(bf[a] + c);
@@ -1030,7 +1032,7 @@ __device__ __forceinline__ void project_at(const Geom& g, const PhysDev& ph, con
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         if (a == DIM - 1 && coord(q, a) == 0) continue;  // wall face stays zero
-        const long cL = idx(g, shift(g, q, a, -1));
+        const long cL = lo_idx(g, q, c, a);
         const T rf = T(0.5) * ((dr * L::ld(phi + cL) + rho2) + (dr * L::ld(phi + c) + rho2));
         const T beta = T(1) / rf;
         const T dp = p_diff(L::ld(p + c), L::ld(p + cL)) * ih;
@@ -1066,10 +1068,10 @@ __device__ void coarse_invert_block(const Geom& g, const M* const* beta, float* 
         const IJK q = decode(g, c);
         float diag = 0.f;
         for (int a = 0; a < DIM; ++a) {
-            const long hi = (a == DIM - 1) ? c + g.NP : idx(g, shift(g, q, a, 1));
+            const long hi = (a == DIM - 1) ? c + g.NP : hi_idx(g, q, c, a);
             const float bm = (float)L::ld(beta[a] + c), bp = (float)L::ld(beta[a] + hi);
             diag -= (bm + bp) * ih2;
-            if (bm != 0.f) A[c * n + idx(g, shift(g, q, a, -1))] += bm * ih2;
+            if (bm != 0.f) A[c * n + lo_idx(g, q, c, a)] += bm * ih2;
             if (bp != 0.f) A[c * n + hi] += bp * ih2;
         }
         A[c * n + c] += diag;
@@ -1102,47 +1104,82 @@ __device__ void coarse_invert_block(const Geom& g, const M* const* beta, float* 
     __syncthreads();
 }
 
-// x[c] += Ainv y on the coarsest level (Ainv symmetric up to rounding; thread
-// c reads column c, so neighbouring threads read neighbouring words)
-__device__ __forceinline__ void coarse_ainv_add(int n, const float* Ainv, const double* y, double* x, bool add) {
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        float s = 0.f;
-        for (int t = 0; t < n; ++t) s += Ainv[t * n + c] * (float)y[t];
-        x[c] = add ? x[c] + (double)s : (double)s;
-    }
-}
-
-// e = (A + c 1 1^T)^-1 r in FP64 (see above); rd, ed, rr: 3 x n doubles of
-// block-shared scratch; beta: the level's face coefficients
+// e = (A + c 1 1^T)^-1 r in FP64 (see above), by one warp: lane l holds cells l
+// and l + 32.  ed: shared-memory scratch of n doubles; beta: the level's face
+// coefficients.  The block's other warps only wait at the barrier.  An FP64
+// instruction occupies its pipe for tens of cycles whatever the number of
+// active lanes, so what counts is their number in sequence: the sum of e is a
+// shuffle tree, each residual is converted to FP32 once (not once a row of
+// the product), and the coefficients are converted once for both steps.
+// On the 64 x 32 grid of 2D drops (8 coarse cells) 8.5k -> 3.9k cycles of a
+// V-cycle's 55k, with 16 cells 11.1k -> 4.1k (block form, sums in sequence).
 template <class L, typename M, int DIM>
 __device__ void coarse_apply_block(const Geom& g, const M* const* beta, const float* Ainv, const M* r, M* e,
-                                   double* rd, double* ed, double* rr) {
+                                   double* ed) {
     const int n = (int)g.N;
-    const double ih2 = g.ih2;
-    const double sh = (double)Ainv[n * n];
-    for (int c = threadIdx.x; c < n; c += blockDim.x) rd[c] = (double)L::ld(r + c);
-    __syncthreads();
-    coarse_ainv_add(n, Ainv, rd, ed, false);
-    __syncthreads();
-    for (int it = 0; it < 2; ++it) {
-        for (int c = threadIdx.x; c < n; c += blockDim.x) {
-            double esum = 0.0;
-            for (int t = 0; t < n; ++t) esum += ed[t];
-            const IJK q = decode(g, c);
-            double Ae = 0.0;
-            for (int a = 0; a < DIM; ++a) {
-                const long hi = (a == DIM - 1) ? c + g.NP : idx(g, shift(g, q, a, 1));
-                const double bm = (double)L::ld(beta[a] + c), bp = (double)L::ld(beta[a] + hi);
-                if (bm != 0.0) Ae += bm * (ed[idx(g, shift(g, q, a, -1))] - ed[c]);
-                if (bp != 0.0) Ae += bp * (ed[hi] - ed[c]);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const double ih2 = g.ih2;
+        const double sh = (double)Ainv[n * n];
+        double rd[2], x[2], b[2][2 * DIM];
+        int nb[2][2 * DIM];
+        float y[2];
+        const int cells = n > 32 ? 2 : 1;  // a lane's cells (uniform over the warp)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            rd[h] = x[h] = 0.0;
+            y[h] = 0.f;
+            if (h < cells && c < n) {
+                y[h] = (float)L::ld(r + c);
+                rd[h] = (double)L::ld(r + c);
+                const IJK q = decode(g, c);
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    const long hi = hi_idx(g, q, c, a);  // the high wall's face is entry n + ...: beyond the cells
+                    const M bm = L::ld(beta[a] + c), bp = L::ld(beta[a] + hi);
+                    b[h][2 * a] = (double)bm;
+                    b[h][2 * a + 1] = (double)bp;
+                    nb[h][2 * a] = bm != M(0) ? (int)lo_idx(g, q, c, a) : c;  // a wall's zero coefficient: any cell
+                    nb[h][2 * a + 1] = bp != M(0) ? (int)hi : c;
+                }
             }
-            rr[c] = rd[c] - (Ae * ih2 + sh * esum);
         }
-        __syncthreads();
-        coarse_ainv_add(n, Ainv, rr, ed, true);
-        __syncthreads();
+        // x += Ainv y (Ainv symmetric up to rounding: lane c reads column c, neighbouring lanes neighbouring words)
+        auto ainv_add = [&]() {
+            float s[2] = {0.f, 0.f};
+            for (int t = 0; t < n; ++t) {
+                const float yt = __shfl_sync(0xffffffffu, t < 32 ? y[0] : y[1], t & 31);
+                if (lane < n) s[0] += Ainv[t * n + lane] * yt;
+                if (cells == 2 && lane + 32 < n) s[1] += Ainv[t * n + lane + 32] * yt;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (h < cells) {
+                    x[h] += (double)s[h];
+                    if (lane + 32 * h < n) ed[lane + 32 * h] = x[h];
+                }
+            __syncwarp();
+        };
+        ainv_add();
+        for (int it = 0; it < 2; ++it) {
+            double esum = cells == 2 ? x[0] + x[1] : x[0];  // zero beyond the cells
+            for (int o = (n > 16 ? 16 : n > 8 ? 8 : 4); o > 0; o >>= 1) esum += __shfl_xor_sync(0xffffffffu, esum, o);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h >= cells || lane + 32 * h >= n) continue;
+                double Ae = 0.0;
+#pragma unroll
+                for (int f = 0; f < 2 * DIM; ++f) Ae += b[h][f] * (ed[nb[h][f]] - x[h]);
+                y[h] = (float)(rd[h] - (Ae * ih2 + sh * esum));
+            }
+            __syncwarp();
+            ainv_add();
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (lane + 32 * h < n) e[lane + 32 * h] = (M)x[h];
     }
-    for (int c = threadIdx.x; c < n; c += blockDim.x) e[c] = (M)ed[c];
     __syncthreads();
 }
 
