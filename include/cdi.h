@@ -256,7 +256,10 @@ cdi_status cdi_set_level0_sweep(cdi_ctx* ctx, int mode);
 
 /* Longest wait (nanoseconds, 0 .. 6e10; default 2e9) of a grid barrier in the
  * persistent step kernel before the call ends with CDI_ETIMEOUT.  A timed-out
- * call leaves the state undefined but the context and the device usable. */
+ * call leaves the state undefined but the context and the device usable.
+ * Grids of up to 4096 cells (FP64) or 8192 (FP32-mixed) step on one cluster,
+ * whose hardware barriers need no limit, unless a limit other than the
+ * default is set here. */
 cdi_status cdi_set_barrier_timeout(cdi_ctx* ctx, long long ns);
 
 /* Launch profiler (diagnostics): from now on record a CUDA event pair on the

@@ -24,6 +24,8 @@
 
 using namespace cdi;
 
+constexpr long kSpinLimit = 2000000000L;  // default barrier timeout
+
 struct cdi_ctx {
     Geom g{};
     double L[3] = {0, 0, 0};
@@ -71,7 +73,7 @@ struct cdi_ctx {
     int exec = CDI_EXEC_AUTO;
     PersistCtl* ctl = nullptr;
     bool persist_ready = false;
-    void* tail_dev = nullptr;  // launch-per-kernel path: descriptor of the V-cycle's shared-memory tail
+    InstArgs<float> tail{};    // launch-per-kernel path: descriptor of the V-cycle's shared-memory tail
     bool tail_ready = false;
     SweepMaps smaps{};         // tensor maps of the one-pass sweep (encoded with the tail)
     // launch-per-kernel path: one V-cycle plus its residual norm as a CUDA graph per form
@@ -95,7 +97,8 @@ struct cdi_ctx {
     int persist_lt = 0;
     size_t persist_smem = 0;
     int persist_grid = 0;
-    long spin_limit_ns = 2000000000L;
+    int persist_cluster = 0;
+    long spin_limit_ns = kSpinLimit;
     // statistics
     int last_cycles = 0;
     double last_resid = 0.0;
@@ -209,7 +212,6 @@ void carve(cdi_ctx* c, char* base, size_t* total) {
     mg.scalf = (float*)cv.take(SF_NSCAL * sizeof(float));
     mg.ainv = (float*)cv.take(((size_t)kMaxCoarse * kMaxCoarse + 1) * sizeof(float));  // inverse, then the shift
     c->ctl = (PersistCtl*)cv.take(sizeof(PersistCtl));
-    c->tail_dev = cv.take(sizeof(InstArgs<float>));
     for (int k = 0; k < 4; ++k)
         for (int j = 0; j < 2; ++j) c->hist[k][j] = (double*)cv.take((size_t)g.N * sizeof(double));
     *total = cv.off + 256;
@@ -398,7 +400,7 @@ cdi_status kernels_tail_setup(cdi_ctx* c) {
     const size_t sm = pick_tail(c, budget, &lt, &lay, kTailMaxCells);
     c->mg.tail_args = nullptr;
     if (sm <= budget) {
-        InstArgs<float> A{};
+        InstArgs<float>& A = c->tail;
         static_cast<PersistLayout&>(A) = lay;
         A.g = c->g;
         for (int l = 0; l < kMaxLevels; ++l) A.lv[l] = c->mg.lv[l];
@@ -408,14 +410,9 @@ cdi_status kernels_tail_setup(cdi_ctx* c) {
         A.npost = c->npost;
         A.ainv = c->mg.ainv;
         A.tail_bf_stored = 1;  // launch_mg_coef restricts the coefficients of every level once per solve
-        st = cuda_check(c, cudaMemcpyAsync(c->tail_dev, &A, sizeof A, cudaMemcpyHostToDevice, c->stream),
-                        "cudaMemcpyAsync(tail)");
-        if (st) return st;
-        st = cuda_check(c, cudaStreamSynchronize(c->stream), "tail setup");
-        if (st) return st;
         st = cuda_check(c, tail_prepare(c->g.D, sm), "tail kernel setup");
         if (st) return st;
-        c->mg.tail_args = c->tail_dev;
+        c->mg.tail_args = &c->tail;
         c->mg.tail_lt = lt;
         c->mg.tail_smem = sm;
     }
@@ -796,7 +793,8 @@ cdi_status persist_setup(cdi_ctx* c) {
     if (st) return st;
     const size_t budget = optin > 8192 ? optin - 4096 : 0;
     c->persist_smem = pick_tail(c, budget, &c->persist_lt, &c->playout);
-    st = cuda_check(c, persist_prepare<T>(c->g.D, c->persist_smem, &c->persist_grid), "persistent kernel setup");
+    st = cuda_check(c, persist_prepare<T>(c->g.D, c->persist_smem, &c->persist_grid, &c->persist_cluster),
+                    "persistent kernel setup");
     if (st) return st;
     c->persist_ready = true;
     return CDI_OK;
@@ -881,8 +879,11 @@ cdi_status step_persist(cdi_ctx* c, double dt, int nsteps) {
     st = cuda_check(c, cudaMemsetAsync(c->ctl, 0, sizeof(PersistCtl), c->stream), "cudaMemsetAsync(ctl)");
     if (st) return st;
     const bool on = prof_before(KC_STEP, c->stream);
-    st = cuda_check(c, launch_step_persist<T>(A, c->persist_smem, c->persist_grid, c->stream),
-                    "cudaLaunchCooperativeKernel");
+    // one cluster for grids of up to about a cell a thread (half a cell in FP64, whose pipes 16 SMs share); a caller
+    // who sets the barrier timeout gets the kernel whose barriers have one
+    const bool small = c->g.N <= (sizeof(T) == 8 ? 4096 : 8192) && c->spin_limit_ns == kSpinLimit;
+    st = cuda_check(c, launch_step_persist<T>(A, c->persist_smem, c->persist_grid, small ? c->persist_cluster : 0,
+                                              c->stream), "persistent step launch");
     prof_after(on, c->stream);
     if (st) return st;
     ++g_launches;

@@ -241,6 +241,8 @@ struct MGLevel {
     float* bf[3];
 };
 
+template <typename T> struct InstArgs;
+
 struct MG {
     int nlev;
     MGLevel lv[kMaxLevels];
@@ -249,9 +251,9 @@ struct MG {
     float* scalf;       // FP32 device scalars
     float* ainv;        // launch-per-kernel path: FP32 inverse of the coarsest level [n^2] and its shift
     // launch-per-kernel path: levels tail_lt .. nlev-1 of a V-cycle run as one
-    // single-CTA launch in shared memory (tail_args: its descriptor in device
-    // memory, an InstArgs<float>; null: every level as separate kernels)
-    const void* tail_args;
+    // single-CTA launch in shared memory (tail_args: its descriptor, copied
+    // into the launch; null: every level as separate kernels)
+    const InstArgs<float>* tail_args;
     int tail_lt;
     size_t tail_smem;
     // launch-per-kernel path, 3D level 0: 0 one-pass sweeps where the grid
@@ -349,7 +351,7 @@ cudaError_t resid_tile_prepare();
 unsigned launch_resid_tile(const MGLevel& L0, const float* fmean_df, double* part, int max_parts, cudaStream_t s);
 // the single-CTA shared-memory tail of a V-cycle as its own launch (k_persist.cu)
 cudaError_t tail_prepare(int dim, size_t smem);
-cudaError_t launch_tail(const void* inst_args, int dim, size_t smem, cudaStream_t s);
+cudaError_t launch_tail(const InstArgs<float>& A, int dim, size_t smem, cudaStream_t s);
 // host <-> level-0 p / f conversions of the FP32-mixed form (FP64 staging buffer x)
 void launch_p_to_double(const Geom& g, const MG& mg, double* x, cudaStream_t s);
 void launch_p_from_double(const Geom& g, MG& mg, const double* x, cudaStream_t s);
@@ -443,9 +445,9 @@ struct BatchArgs {
 
 size_t persist_tail_layout(const Geom& g, const MG& mg, int lt, PersistLayout& L);
 template <typename T>
-cudaError_t persist_prepare(int dim, size_t smem, int* grid);
+cudaError_t persist_prepare(int dim, size_t smem, int* grid, int* cluster);  // cluster: its CTAs, 0 if none fits
 template <typename T>
-cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, cudaStream_t s);
+cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, int cluster, cudaStream_t s);
 template <typename T>
 cudaError_t batch_prepare(int dim, int threads, size_t smem, int cluster, int* groups);  // groups: CTAs or clusters resident at once
 template <typename T>

@@ -1071,7 +1071,7 @@ template <typename T, int DIM>
 static bool vcycle_rec(MG& mg, PT<T>* p, int l, int npre, int npost, cudaStream_t s) {
     MGLevel& L = mg.lv[l];
     if (mg.tail_args && l == mg.tail_lt) {
-        CDI_PROF(KC_COARSE, s, launch_tail(mg.tail_args, DIM, mg.tail_smem, s));
+        CDI_PROF(KC_COARSE, s, launch_tail(*mg.tail_args, DIM, mg.tail_smem, s));
         ++g_launches;
         return false;
     }

@@ -115,7 +115,9 @@ struct GridX {
     // Grid barrier on one arrival counter that only grows: barrier number m
     // is passed once the counter reaches m x gridDim.x.  Thread 0 arrives with
     // one acquire-release atomic (publishing the CTA's writes, ordered before
-    // it by __syncthreads) and polls with acquire loads.  A wait longer than
+    // it by __syncthreads) and polls with acquire loads.  (A release reduction
+    // and polls without a pause made the 512 x 128 step 3 % slower: the polls
+    // delay the arrivals.)  A wait longer than
     // `limit` ns (or 2^31 polls) sets CDI_ETIMEOUT and sets the bit kBarError
     // of the counter with an atomic OR (idempotent, so CTAs that give up at
     // the same time cannot carry it out of the word; arrivals never reach
@@ -729,6 +731,20 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_step_persist(PersistArgs
     run_steps<T, DIM>(P.I, x, P.nsteps, &P.ctl->st, sm);
 }
 
+// k_step_persist on one cluster, for grids of about its threads (cdi_api.cu
+// step_persist): their phases are bound by latency on any number of SMs, and a
+// hardware cluster barrier takes a fraction of the grid barrier's 1.2 us.
+// A step on the grid / on the cluster (ms): 64 x 32 FP64 0.97 / 0.86, FP32-mixed
+// 0.55 / 0.47; 128 x 64 FP32-mixed 0.83 / 0.76; 32 x 16 FP64 0.81 / 0.68.
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kPersistThreads, 1) k_step_cluster(PersistArgs<T> P) {
+    extern __shared__ double smd[];
+    __shared__ double s_slots[2 * kMaxCluster];
+    ClusterX x{ClusterX::cluster_rank(), ClusterX::cluster_size(), s_slots, 0};
+    run_steps<T, DIM>(P.I, x, P.nsteps, &P.ctl->st, reinterpret_cast<float*>(smd));
+    ClusterX::cluster_barrier();  // no CTA ends while another may still write to its shared memory
+}
+
 template <typename T, int DIM, int NT>
 __global__ void __launch_bounds__(NT, 1) k_batch_persist(BatchArgs<T> B) {
     extern __shared__ double smd[];
@@ -807,11 +823,40 @@ size_t persist_tail_layout(const Geom& g, const MG& mg, int lt, PersistLayout& L
 
 // One V-cycle's shared-memory tail as its own single-CTA launch (the
 // launch-per-kernel path): levels lt .. nlev-1 of the descriptor, the tail
-// coefficients restricted afresh each launch (shared memory does not outlive it)
+// coefficients restricted afresh each launch (shared memory does not outlive
+// it).  The descriptor is a kernel parameter: read from global memory, every
+// phase waited for its level's geometry.
 template <int DIM>
-__global__ void __launch_bounds__(kPersistThreads, 1) k_tail(const InstArgs<float>* A) {
+__global__ void __launch_bounds__(kPersistThreads, 1) k_tail(const __grid_constant__ InstArgs<float> A) {
     extern __shared__ double smd[];
-    tail_vcycle<float, DIM>(*A, true, reinterpret_cast<float*>(smd));
+    tail_vcycle<float, DIM>(A, true, reinterpret_cast<float*>(smd));
+}
+
+static void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, int clusters, int threads,
+                                  size_t smem, cudaStream_t s) {
+    cfg.gridDim = dim3((unsigned)(cluster * clusters));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)cluster, 1, 1};
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+// the largest cluster (16 or 8 CTAs) of fn that the device can hold with this shared memory, or 0
+static int largest_cluster(const void* fn, int threads, size_t smem) {
+    for (int n = kMaxCluster; n >= 8; n /= 2) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cluster_config(cfg, at, n, 1, threads, smem, nullptr);
+        int fit = 0;
+        if ((n <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+            cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) == cudaSuccess && fit >= 1)
+            return n;
+        cudaGetLastError();
+    }
+    return 0;
 }
 
 cudaError_t tail_prepare(int dim, size_t smem) {
@@ -819,22 +864,28 @@ cudaError_t tail_prepare(int dim, size_t smem) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-cudaError_t launch_tail(const void* inst_args, int dim, size_t smem, cudaStream_t s) {
-    const InstArgs<float>* A = static_cast<const InstArgs<float>*>(inst_args);
+cudaError_t launch_tail(const InstArgs<float>& A, int dim, size_t smem, cudaStream_t s) {
     if (dim == 2) k_tail<2><<<1, kPersistThreads, smem, s>>>(A);
     else k_tail<3><<<1, kPersistThreads, smem, s>>>(A);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, cudaStream_t s) {
+cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, int cluster, cudaStream_t s) {
     void* args[] = {&A};
+    if (cluster) {
+        const void* fn = (A.I.g.D == 2) ? (const void*)k_step_cluster<T, 2> : (const void*)k_step_cluster<T, 3>;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cluster_config(cfg, at, cluster, 1, kPersistThreads, smem, s);
+        return cudaLaunchKernelExC(&cfg, fn, args);
+    }
     const void* fn = (A.I.g.D == 2) ? (const void*)k_step_persist<T, 2> : (const void*)k_step_persist<T, 3>;
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPersistThreads), args, smem, s);
 }
 
 template <typename T>
-cudaError_t persist_prepare(int dim, size_t smem, int* grid) {
+cudaError_t persist_prepare(int dim, size_t smem, int* grid, int* cluster) {
     const void* fn = (dim == 2) ? (const void*)k_step_persist<T, 2> : (const void*)k_step_persist<T, 3>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -844,6 +895,12 @@ cudaError_t persist_prepare(int dim, size_t smem, int* grid) {
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kPersistThreads, smem)) != cudaSuccess) return e;
     if (per < 1) return cudaErrorInvalidConfiguration;
     *grid = nsm;  // one CTA per SM
+    fn = (dim == 2) ? (const void*)k_step_cluster<T, 2> : (const void*)k_step_cluster<T, 3>;
+    *cluster = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
+        *cluster = largest_cluster(fn, kPersistThreads, smem);
+    else
+        cudaGetLastError();
     return cudaSuccess;
 }
 
@@ -875,13 +932,7 @@ cudaError_t batch_prepare(int dim, int threads, size_t smem, int cluster, int* g
             return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at{};
-        cfg.gridDim = dim3(nsm / cluster * cluster);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim = {(unsigned)cluster, 1, 1};
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
+        cluster_config(cfg, at, cluster, nsm / cluster, threads, smem, nullptr);
         if ((e = cudaOccupancyMaxActiveClusters(&per, fn, &cfg)) != cudaSuccess) return e;
         if (per < 1) return cudaErrorInvalidConfiguration;
         *groups = per;
@@ -901,21 +952,14 @@ cudaError_t launch_batch_persist(BatchArgs<T>& B, int dim, int threads, size_t s
     if (cluster == 1) return cudaLaunchKernel(fn, dim3(groups), dim3(threads), args, smem, s);
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
-    cfg.gridDim = dim3((unsigned)(groups * cluster));
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim = {(unsigned)cluster, 1, 1};
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cluster_config(cfg, at, cluster, groups, threads, smem, s);
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-template cudaError_t launch_step_persist<double>(PersistArgs<double>&, size_t, int, cudaStream_t);
-template cudaError_t launch_step_persist<float>(PersistArgs<float>&, size_t, int, cudaStream_t);
-template cudaError_t persist_prepare<double>(int, size_t, int*);
-template cudaError_t persist_prepare<float>(int, size_t, int*);
+template cudaError_t launch_step_persist<double>(PersistArgs<double>&, size_t, int, int, cudaStream_t);
+template cudaError_t launch_step_persist<float>(PersistArgs<float>&, size_t, int, int, cudaStream_t);
+template cudaError_t persist_prepare<double>(int, size_t, int*, int*);
+template cudaError_t persist_prepare<float>(int, size_t, int*, int*);
 template cudaError_t batch_prepare<double>(int, int, size_t, int, int*);
 template cudaError_t batch_prepare<float>(int, int, size_t, int, int*);
 template cudaError_t launch_batch_persist<double>(BatchArgs<double>&, int, int, size_t, int, int, cudaStream_t);
