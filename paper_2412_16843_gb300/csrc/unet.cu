@@ -296,17 +296,27 @@ __global__ void k_loss(int N, const float* y, const float* t, bf16* gy, float* p
     if (threadIdx.x == 0) atomicAdd(part, sh[0]);
 }
 
+// the parameter arrays of the network, one segment each, for one launch over all of them (16 launches of a few
+// microseconds each otherwise)
+struct ParamSegs {
+    long end[2 * kLayers];  // running ends of the segments
+    float *w[2 * kLayers], *g[2 * kLayers], *m[2 * kLayers], *v[2 * kLayers];
+};
+
 // Adam (Kingma and Ba, 2015) with bias corrections bc1 = 1 - b1^t, bc2 = 1 - b2^t
-__global__ void k_adam(long n, float* w, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
-                       float bc1, float bc2) {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+__global__ void k_adam(const __grid_constant__ ParamSegs p, float lr, float b1, float b2, float eps, float bc1,
+                       float bc2) {
+    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.end[2 * kLayers - 1]) return;
+    int k = 0;
+    while (i >= p.end[k]) ++k;
+    if (k) i -= p.end[k - 1];
+    const float gi = p.g[k][i];
+    const float mi = b1 * p.m[k][i] + (1.f - b1) * gi;
+    const float vi = b2 * p.v[k][i] + (1.f - b2) * gi * gi;
+    p.m[k][i] = mi;
+    p.v[k][i] = vi;
+    p.w[k][i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
 // output channels of one CTA of the tcgen05 convolution with n output channels
@@ -321,21 +331,32 @@ __device__ __forceinline__ size_t conv_w_at(int t, int o, int n, int i, int cin)
     return (blk * 9 + t % 9) * (3 * NB * 16) + (row >> 3) * 128 + ((i >> 3) & 1) * 64 + (row & 7) * 8 + (i & 7);
 }
 
+// the weights of every layer and their BF16 copies, one segment a layer (padded elements)
+struct WeightSegs {
+    long end[kLayers];
+    const float* W[kLayers];
+    int taps[kLayers], cout[kLayers], cin[kLayers], co_pad[kLayers], ci_pad[kLayers];
+    bf16 *wb[kLayers], *wt[kLayers], *wk[kLayers], *wkt[kLayers];
+};
+
 // BF16 copies: wb[t][co_pad][ci_pad] = W[t][co][ci]; wt[t][ci_pad][co_pad] = W[T-1-t][co][ci]; for 27 taps
 // also both in the order of the tcgen05 convolution (wk, wkt)
-__global__ void k_weights_bf16(const float* W, int taps, int cout, int cin, int co_pad, int ci_pad, bf16* wb,
-                               bf16* wt, bf16* wk, bf16* wkt) {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long n = (long)taps * co_pad * ci_pad;
-    if (i >= n) return;
-    const int ci = (int)(i % ci_pad), co = (int)((i / ci_pad) % co_pad), t = (int)(i / ((long)ci_pad * co_pad));
-    const bf16 val = __float2bfloat16((co < cout && ci < cin) ? W[((size_t)t * cout + co) * cin + ci] : 0.f);
-    wb[i] = val;
+__global__ void k_weights_bf16(const __grid_constant__ WeightSegs p) {
+    long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.end[kLayers - 1]) return;
+    int l = 0;
+    while (i >= p.end[l]) ++l;
+    if (l) i -= p.end[l - 1];
+    const int ci_pad = p.ci_pad[l], co_pad = p.co_pad[l], taps = p.taps[l], cout = p.cout[l], cin = p.cin[l];
+    const unsigned r = (unsigned)i / (unsigned)ci_pad;
+    const int ci = (int)((unsigned)i - r * (unsigned)ci_pad), t = (int)(r / (unsigned)co_pad), co = (int)r - t * co_pad;
+    const bf16 val = __float2bfloat16((co < cout && ci < cin) ? p.W[l][((size_t)t * cout + co) * cin + ci] : 0.f);
+    p.wb[l][i] = val;
     const int tf = taps - 1 - t;
-    wt[((size_t)tf * ci_pad + ci) * co_pad + co] = val;
+    p.wt[l][((size_t)tf * ci_pad + ci) * co_pad + co] = val;
     if (taps == 27) {
-        wk[conv_w_at(t, co, co_pad, ci, ci_pad)] = val;
-        wkt[conv_w_at(tf, ci, ci_pad, co, co_pad)] = val;
+        p.wk[l][conv_w_at(t, co, co_pad, ci, ci_pad)] = val;
+        p.wkt[l][conv_w_at(tf, ci, ci_pad, co, co_pad)] = val;
     }
 }
 
@@ -921,7 +942,7 @@ __global__ void __launch_bounds__(kZbThreads, PAIRS ? 2 : 1) k_conv_zb(const Con
 // memory is released under the same rules as in k_conv_tc.
 // ---------------------------------------------------------------------------
 constexpr int kWgK = 128;        // voxels per chunk
-constexpr int kWgThreads = 128;
+constexpr int kWgThreads = 256;  // staging; the accumulators are read out by the first 128
 constexpr int kWgSbo = 272;      // bytes between the core matrices of consecutive 8-row groups
 constexpr int kWgAStep = 16 * kWgSbo;   // bytes of one K = 16 step of A (16 row groups)
 constexpr int kWgABytes = (kWgK / 16) * kWgAStep;
@@ -997,6 +1018,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
         }
     };
     const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+    const bool rows8 = g.nx % 8 == 0;
     // stage chunk ch0 + c into buffer b
     auto stage = [&](int c, int b) {
         unsigned char* A = smem + b * bufb;
@@ -1011,10 +1033,25 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
                 const int tap = row0 / cin_pad, ci0 = row0 - tap * cin_pad;
                 int dz, dyy, dx;
                 tap_off(tap, ntaps, dz, dyy, dx);
+                if (rows8) {
+                    // the octet lies in one x row: one decode, and only the row's ends can miss a neighbour
+                    const Vox q = vox(g, vbase + 8 * o);
+                    const int y = q.y + dyy, z = q.z + dz;
+                    const bool ok = q.in && y >= 0 && y < g.ny && z >= 0 && z < g.nz;
+                    const uint4* src = reinterpret_cast<const uint4*>(
+                        x + ((ptrdiff_t)((long)(ok ? z : 0) * g.ny + (ok ? y : 0)) * g.nx + q.x + dx) * cin_pad + ci0);
+                    const int step = cin_pad / 8;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int n = nbr(g, vox(g, vbase + 8 * o + e), dz, dyy, dx);
-                    in[e] = n >= 0 ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)n * cin_pad + ci0)) : zero4;
+                    for (int e = 0; e < 8; ++e) {
+                        const int xe = q.x + dx + e;
+                        in[e] = ok && xe >= 0 && xe < g.nx ? __ldg(src + e * step) : zero4;
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int n = nbr(g, vox(g, vbase + 8 * o + e), dz, dyy, dx);
+                        in[e] = n >= 0 ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)n * cin_pad + ci0)) : zero4;
+                    }
                 }
             } else {
                 // the row of ones (channel 0 of the group starting at row R), then zeros
@@ -1070,7 +1107,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
     }
     for (int b = 0; b < 2; ++b) wait_mma(b);
     __syncthreads();
-    if (!s_abort && nch > 0) {
+    if (!s_abort && nch > 0 && warp < 4) {
         tc_fence_after();
         const int row = warp * 32 + lane;
         float* dst = part + ((size_t)(blockIdx.y * nrb + rb) * 128 + row) * N;
@@ -1433,11 +1470,23 @@ void conv_wgrad(cdi_unet* u, int l, const CG& gl, const bf16* in, const bf16* dy
 }
 
 void refresh_weights(cdi_unet* u) {
+    WeightSegs p;
+    long n = 0;
     for (int l = 0; l < kLayers; ++l) {
-        const long n = (long)kTaps[l] * u->co_pad[l] * u->ci_pad[l];
-        k_weights_bf16<<<blocks(n), 256, 0, u->stream>>>(u->W[l], kTaps[l], kCout[l], kCin[l], u->co_pad[l],
-                                                          u->ci_pad[l], u->Wb[l], u->Wt[l], u->Wk[l], u->Wkt[l]);
+        n += (long)kTaps[l] * u->co_pad[l] * u->ci_pad[l];
+        p.end[l] = n;
+        p.W[l] = u->W[l];
+        p.taps[l] = kTaps[l];
+        p.cout[l] = kCout[l];
+        p.cin[l] = kCin[l];
+        p.co_pad[l] = u->co_pad[l];
+        p.ci_pad[l] = u->ci_pad[l];
+        p.wb[l] = u->Wb[l];
+        p.wt[l] = u->Wt[l];
+        p.wk[l] = u->Wk[l];
+        p.wkt[l] = u->Wkt[l];
     }
+    k_weights_bf16<<<blocks(n), 256, 0, u->stream>>>(p);
     u->weights_ready = true;
 }
 
@@ -1481,7 +1530,7 @@ void forward(cdi_unet* u, bool keep, float* y) {
 void backward(cdi_unet* u) {
     const CG* g = u->g;
     cudaStream_t s = u->stream;
-    for (int l = 0; l < kLayers; ++l) {
+    for (int l = 0; l < kLayers && !u->wgrad_tc; ++l) {  // summed with atomics (the tcgen05 form stores every entry)
         cudaMemsetAsync(u->gW[l], 0, (size_t)kTaps[l] * kCout[l] * kCin[l] * 4, s);
         cudaMemsetAsync(u->gB[l], 0, (size_t)kCout[l] * 4, s);
     }
@@ -1534,13 +1583,16 @@ void adam(cdi_unet* u, double lr) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float bc1 = (float)(1.0 - std::pow(0.9, (double)u->adam_t));
     const float bc2 = (float)(1.0 - std::pow(0.999, (double)u->adam_t));
+    ParamSegs p;
+    long n = 0;
     for (int l = 0; l < kLayers; ++l) {
-        const long nw = (long)kTaps[l] * kCout[l] * kCin[l];
-        k_adam<<<blocks(nw), 256, 0, u->stream>>>(nw, u->W[l], u->gW[l], u->mW[l], u->vW[l], (float)lr, b1, b2, eps,
-                                                   bc1, bc2);
-        k_adam<<<blocks(kCout[l]), 256, 0, u->stream>>>(kCout[l], u->B[l], u->gB[l], u->mB[l], u->vB[l], (float)lr,
-                                                         b1, b2, eps, bc1, bc2);
+        const int i = 2 * l;
+        p.end[i] = n += (long)kTaps[l] * kCout[l] * kCin[l];
+        p.end[i + 1] = n += kCout[l];
+        p.w[i] = u->W[l]; p.g[i] = u->gW[l]; p.m[i] = u->mW[l]; p.v[i] = u->vW[l];
+        p.w[i + 1] = u->B[l]; p.g[i + 1] = u->gB[l]; p.m[i + 1] = u->mB[l]; p.v[i + 1] = u->vB[l];
     }
+    k_adam<<<blocks(n), 256, 0, u->stream>>>(p, (float)lr, b1, b2, eps, bc1, bc2);
     refresh_weights(u);
 }
 
