@@ -222,15 +222,22 @@ __global__ void k_pool(CG gf, const bf16* in, int C, bf16* out) {
     *reinterpret_cast<uint4*>(out + (size_t)V * C + 8 * g8) = *reinterpret_cast<const uint4*>(o);
 }
 
-// din[v][off+c] += dout[parent(v)][c] / 8 on the fine grid gf
+// din[v][off+c] += dout[parent(v)][c] / 8 on the fine grid gf; 8 channels (16 bytes) per thread
 __global__ void k_pool_bwd_add(CG gf, const bf16* dout, int C, bf16* din, int stride, int off) {
+    const int C8 = C / 8;
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)gf.N * C) return;
-    const int c = (int)(t % C), v = (int)(t / C);
+    if (t >= (long)gf.N * C8) return;
+    const int g8 = (int)(t % C8), v = (int)(t / C8);
     const int x = v % gf.nx, y = (v / gf.nx) % gf.ny, z = v / (gf.nx * gf.ny);
     const int P = (x / 2) + (gf.nx / 2) * ((y / 2) + (gf.ny / 2) * (z / 2));
-    const size_t o = (size_t)v * stride + off + c;
-    din[o] = __float2bfloat16(__bfloat162float(din[o]) + 0.125f * __bfloat162float(dout[(size_t)P * C + c]));
+    uint4* dst = reinterpret_cast<uint4*>(din + (size_t)v * stride + off + 8 * g8);
+    uint4 d = *dst;
+    const uint4 q = *reinterpret_cast<const uint4*>(dout + (size_t)P * C + 8 * g8);
+    bf16* a = reinterpret_cast<bf16*>(&d);
+    const bf16* h = reinterpret_cast<const bf16*>(&q);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) a[e] = __float2bfloat16(__bfloat162float(a[e]) + 0.125f * __bfloat162float(h[e]));
+    *dst = d;
 }
 
 // nearest upsampling of the coarse input into channels [off, off+C) of the fine output; 8 channels per thread
@@ -272,10 +279,18 @@ __global__ void k_copy_ch(int N, const bf16* src, int sstride, int soff, bf16* d
         *reinterpret_cast<const uint4*>(src + (size_t)v * sstride + soff + 8 * g8);
 }
 
-// g *= (y > 0) (ReLU backward), both [N][C] contiguous
+// g *= (y > 0) (ReLU backward), both n contiguous values, a multiple of 8; 8 per thread
 __global__ void k_relu_mask(long n, bf16* g, const bf16* y) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n && !(__bfloat162float(y[t]) > 0.f)) g[t] = __float2bfloat16(0.f);
+    if (8 * t >= n) return;
+    uint4 d = reinterpret_cast<const uint4*>(g)[t];
+    const uint4 q = reinterpret_cast<const uint4*>(y)[t];
+    bf16* a = reinterpret_cast<bf16*>(&d);
+    const bf16* h = reinterpret_cast<const bf16*>(&q);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        if (!(__bfloat162float(h[e]) > 0.f)) a[e] = __float2bfloat16(0.f);
+    reinterpret_cast<uint4*>(g)[t] = d;
 }
 
 // mean squared error: partial sums of (y-t)^2 and the BF16 gradient 2(y-t)/N in channel 0 of 16
@@ -939,7 +954,11 @@ __global__ void __launch_bounds__(kZbThreads, PAIRS ? 2 : 1) k_conv_zb(const Con
 // kWgSbo = 272 bytes apart (not 256), so the eight threads of a store phase
 // hit different bank groups.  Chunks are double-buffered: the MMAs of one
 // chunk run while the next one is staged.  Waits are bounded and tensor
-// memory is released under the same rules as in k_conv_tc.
+// memory is released under the same rules as in k_conv_zb.  Staging is bound by
+// its index arithmetic and load latency: where nx is a multiple of 8 an octet of
+// voxels lies in one row and is decoded once, and 256 threads load a chunk in
+// one round (48 -> 16 layer at 64^3: 412 -> 203 us; a decode a voxel, 128
+// threads and two rounds before).
 // ---------------------------------------------------------------------------
 constexpr int kWgK = 128;        // voxels per chunk
 constexpr int kWgThreads = 256;  // staging; the accumulators are read out by the first 128
@@ -1137,8 +1156,18 @@ __global__ void k_wgrad_reduce(const float* __restrict__ part, int nsplit, int n
     const int n = (int)(t % cout);
     const int m = (int)(t / cout);  // row, 0 .. R
     const int rb = m >> 7, row = m & 127;
+    // added in split order, sixteen loads in flight (the head has 304 splits for 17 outputs: 47 us one at a time)
     float s = 0.f;
-    for (int k = 0; k < nsplit; ++k) s += part[((size_t)(k * nrb + rb) * 128 + row) * N + n];
+    const float* src = part + ((size_t)rb * 128 + row) * N + n;
+    const size_t step = (size_t)nrb * 128 * N;
+    for (int k0 = 0; k0 < nsplit; k0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = k0 + u < nsplit ? __ldg(src + (k0 + u) * step) : 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+            if (k0 + u < nsplit) s += v[u];
+    }
     if (m == R) {
         dB[n] = s;
         return;
@@ -1540,39 +1569,39 @@ void backward(cdi_unet* u) {
     // head and d0
     conv_wgrad(u, 7, g[0], u->d0, u->gy);
     conv_dgrad(u, 7, g[0], u->gy, u->gd0);
-    k_relu_mask<<<blocks(g[0].N * 16L), 256, 0, s>>>(g[0].N * 16L, u->gd0, u->d0);
+    k_relu_mask<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0].N * 16L, u->gd0, u->d0);
     conv_wgrad(u, 6, g[0], u->c0, u->gd0);
     conv_dgrad(u, 6, g[0], u->gd0, u->gc0);
     k_up_bwd<<<blocks(g[1].N * 32L), 256, 0, s>>>(g[0], u->gc0, 48, 0, 32, u->gd1);
-    k_relu_mask<<<blocks(g[1].N * 32L), 256, 0, s>>>(g[1].N * 32L, u->gd1, u->d1);
+    k_relu_mask<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1].N * 32L, u->gd1, u->d1);
     k_copy_ch<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0].N, u->gc0, 48, 32, u->ge0, 16, 0, 16);
     // d1
     conv_wgrad(u, 5, g[1], u->c1, u->gd1);
     conv_dgrad(u, 5, g[1], u->gd1, u->gc1);
     k_up_bwd<<<blocks(g[2].N * 64L), 256, 0, s>>>(g[1], u->gc1, 96, 0, 64, u->gd2);
-    k_relu_mask<<<blocks(g[2].N * 64L), 256, 0, s>>>(g[2].N * 64L, u->gd2, u->d2);
+    k_relu_mask<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2].N * 64L, u->gd2, u->d2);
     k_copy_ch<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1].N, u->gc1, 96, 64, u->ge1, 32, 0, 32);
     // d2
     conv_wgrad(u, 4, g[2], u->c2, u->gd2);
     conv_dgrad(u, 4, g[2], u->gd2, u->gc2);
     k_up_bwd<<<blocks(g[3].N * 128L), 256, 0, s>>>(g[2], u->gc2, 192, 0, 128, u->gb);
-    k_relu_mask<<<blocks(g[3].N * 128L), 256, 0, s>>>(g[3].N * 128L, u->gb, u->b);
+    k_relu_mask<<<blocks(g[3].N * 16L), 256, 0, s>>>(g[3].N * 128L, u->gb, u->b);
     k_copy_ch<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2].N, u->gc2, 192, 128, u->ge2, 64, 0, 64);
     // bottleneck
     conv_wgrad(u, 3, g[3], u->p2, u->gb);
     conv_dgrad(u, 3, g[3], u->gb, u->gp2);
-    k_pool_bwd_add<<<blocks(g[2].N * 64L), 256, 0, s>>>(g[2], u->gp2, 64, u->ge2, 64, 0);
-    k_relu_mask<<<blocks(g[2].N * 64L), 256, 0, s>>>(g[2].N * 64L, u->ge2, u->e2);
+    k_pool_bwd_add<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2], u->gp2, 64, u->ge2, 64, 0);
+    k_relu_mask<<<blocks(g[2].N * 8L), 256, 0, s>>>(g[2].N * 64L, u->ge2, u->e2);
     // e2
     conv_wgrad(u, 2, g[2], u->p1, u->ge2);
     conv_dgrad(u, 2, g[2], u->ge2, u->gp1);
-    k_pool_bwd_add<<<blocks(g[1].N * 32L), 256, 0, s>>>(g[1], u->gp1, 32, u->ge1, 32, 0);
-    k_relu_mask<<<blocks(g[1].N * 32L), 256, 0, s>>>(g[1].N * 32L, u->ge1, u->e1);
+    k_pool_bwd_add<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1], u->gp1, 32, u->ge1, 32, 0);
+    k_relu_mask<<<blocks(g[1].N * 4L), 256, 0, s>>>(g[1].N * 32L, u->ge1, u->e1);
     // e1
     conv_wgrad(u, 1, g[1], u->p0, u->ge1);
     conv_dgrad(u, 1, g[1], u->ge1, u->gp0);
-    k_pool_bwd_add<<<blocks(g[0].N * 16L), 256, 0, s>>>(g[0], u->gp0, 16, u->ge0, 16, 0);
-    k_relu_mask<<<blocks(g[0].N * 16L), 256, 0, s>>>(g[0].N * 16L, u->ge0, u->e0);
+    k_pool_bwd_add<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0], u->gp0, 16, u->ge0, 16, 0);
+    k_relu_mask<<<blocks(g[0].N * 2L), 256, 0, s>>>(g[0].N * 16L, u->ge0, u->e0);
     // e0
     conv_wgrad(u, 0, g[0], u->x, u->ge0);
     g_launches += 50;
