@@ -199,7 +199,8 @@ cdi_status cdi_launches_per_step(cdi_ctx* ctx, long* launches);
 
 /* Execution mode of cdi_step: CDI_EXEC_PERSISTENT runs all steps of the call
  * in one cooperative launch with bounded grid barriers (a barrier that waits
- * longer than 2 s ends the call with CDI_ETIMEOUT); CDI_EXEC_KERNELS launches
+ * longer than 2 s ends the call with CDI_ETIMEOUT; the smallest grids run on
+ * one thread-block cluster instead, see cdi_set_barrier_timeout); CDI_EXEC_KERNELS launches
  * every stencil and multigrid kernel separately; CDI_EXEC_AUTO (default)
  * takes the persistent launch for grids up to 2^20 cells, where launch
  * latency dominates, and separate kernels above, where the separate kernels

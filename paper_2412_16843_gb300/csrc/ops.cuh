@@ -1111,8 +1111,9 @@ __device__ void coarse_invert_block(const Geom& g, const M* const* beta, float* 
 // active lanes, so what counts is their number in sequence: the sum of e is a
 // shuffle tree, each residual is converted to FP32 once (not once a row of
 // the product), and the coefficients are converted once for both steps.
-// On the 64 x 32 grid of 2D drops (8 coarse cells) 8.5k -> 3.9k cycles of a
-// V-cycle's 55k, with 16 cells 11.1k -> 4.1k (block form, sums in sequence).
+// With 8 coarse cells (64 x 32 grid) 8.5k -> 6.3k cycles of a V-cycle's 55k,
+// with 16 (512 x 128) 11.3k -> 8.0k of 106k, against the block form with its
+// sums in sequence.
 template <class L, typename M, int DIM>
 __device__ void coarse_apply_block(const Geom& g, const M* const* beta, const float* Ainv, const M* r, M* e,
                                    double* ed) {
