@@ -834,8 +834,7 @@ void fill_inst(const cdi_ctx* c, InstArgs<T>& A, int lt, const PersistLayout& la
     A.npost = c->npost;
     A.gamma_param = c->gamma;
     A.dt = dt;
-    A.inv_cdt[0] = 1.0 / (0.5 * dt);
-    A.inv_cdt[1] = 1.0 / dt;
+    A.inv_dt = 1.0 / dt;
     for (int k = 0; k < 4; ++k)
         for (int j = 0; j < 2; ++j) A.hist[k][j] = c->hist[k][j];
     A.hist_step0 = c->hist_steps;

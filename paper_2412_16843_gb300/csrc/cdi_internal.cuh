@@ -26,10 +26,9 @@ constexpr int kPartials = 1024;     // blocks of the fixed-order reductions
 // of Granlund and Montgomery, "Division by invariant integers using
 // multiplication", 1994).
 struct FastDiv {
-    unsigned d, m;
+    unsigned m;
     int s;
     __host__ void init(unsigned dv) {
-        d = dv;
         s = 0;
         while ((1ull << s) < dv) ++s;
         m = (unsigned)((((1ull << 32) * ((1ull << s) - dv)) / dv) + 1);
@@ -38,7 +37,7 @@ struct FastDiv {
 #ifdef __CUDA_ARCH__
         return (__umulhi(x, m) + x) >> s;
 #else
-        return x / d;
+        return (unsigned)((((unsigned long long)x * m) >> 32) + x) >> s;
 #endif
     }
 };
@@ -414,7 +413,7 @@ struct __align__(16) InstArgs : PersistLayout {
     double tol;
     int max_vcycles, warm, npre, npost;
     double gamma_param, dt;
-    double inv_cdt[2];   // 1 / (c dt) of the projections of stages 0, 1 (c = 1/2) and 2, 3 (c = 1)
+    double inv_dt;       // 1 / dt
     // first guess by extrapolation in time (CDI_WARM_EXTRAP): the pressure of
     // RK stage k of the last two steps, hist[k][s & 1] written at step s
     double* hist[4][2];

@@ -525,7 +525,7 @@ __device__ bool project(const InstArgs<T>& A, X& x, InstStats* S, const T* phi, 
     const MGLevel L0 = A.lv[0];
     PT<T>* P0 = ops::pbuf<T>(L0);
     FT<T>* F0 = ops::fbuf<T>(L0);
-    const T ih = g_ih<T>(g), inv_cdt = (T)(stage < 2 ? A.inv_cdt[0] : A.inv_cdt[1]);  // 1 / cdt
+    const T ih = g_ih<T>(g), inv_cdt = (T)(stage < 2 ? 2.0 * A.inv_dt : A.inv_dt);  // 1 / cdt: c = 1/2, 1/2, 1, 1
     const T* uc[3] = {u[0], u[1], u[2]};
     ops::SumAcc<T> s;
     for (int c = tid; c < (int)g.N; c += nth) {
