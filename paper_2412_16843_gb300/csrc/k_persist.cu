@@ -741,6 +741,9 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_step_cluster(PersistArgs
     extern __shared__ double smd[];
     __shared__ double s_slots[2 * kMaxCluster];
     ClusterX x{ClusterX::cluster_rank(), ClusterX::cluster_size(), s_slots, 0};
+    // every CTA has started before the first store to another's shared memory (with gamma < 0 a step opens with a
+    // reduction, before any other barrier)
+    ClusterX::cluster_barrier();
     run_steps<T, DIM>(P.I, x, P.nsteps, &P.ctl->st, reinterpret_cast<float*>(smd));
     ClusterX::cluster_barrier();  // no CTA ends while another may still write to its shared memory
 }
