@@ -654,6 +654,11 @@ __device__ __forceinline__ bool mbar_wait_role(uint64_t* bar, uint32_t parity, v
     }
     return true;
 }
+// mbar_wait_role of a whole warp whose lanes go on together: a lane may see the phase complete where another, a poll
+// earlier, saw a role give up, and a warp barrier or tcgen05.ld without all 32 lanes never ends
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+    return __all_sync(0xffffffffu, mbar_wait_role(bar, parity, abort_flag, err));
+}
 
 struct ConvArgs {
     CG g;
@@ -889,8 +894,7 @@ __global__ void __launch_bounds__(kZbThreads, PAIRS ? 2 : 1) k_conv_zb(const Con
             origin(item, x0, y0, z0, blk);
             const int gx = x0 + (m & 7), gy = y0 + (m >> 3);
             const bool in2 = gx < g.nx && gy < g.ny;
-            if (!mbar_wait_role(&b_acc[k & 1], (uint32_t)((k >> 1) & 1), &s_abort, a.err)) break;
-            __syncwarp();
+            if (!mbar_wait_warp(&b_acc[k & 1], (uint32_t)((k >> 1) & 1), &s_abort, a.err)) break;
             tc_fence_after();
             const uint32_t acc = lane_base + (uint32_t)((k & 1) * a.zt * NB);
             const size_t v0 = in2 ? ((size_t)z0 * g.ny + gy) * g.nx + gx : 0;
