@@ -815,10 +815,11 @@ __global__ void __launch_bounds__(kZbThreads, PAIRS ? 2 : 1) k_conv_zb(const Con
             fence_proxy_async();
             mbar_arrive(prev);
         }
-        // after an abort the bulk copies in flight are waited for (bounded) before the CTA may end
-        if (pt == 0 && s_abort)
+        // the CTA ends only once its bulk copies have landed (bounded), also where another role gives up after this one
+        // is through
+        if (pt == 0)
             for (int i = max(0, issued - a.nstage); i < issued; ++i)
-                mbar_drain(&b_wfull[i % a.nstage], (uint32_t)(i / a.nstage) & 1u);
+                if (!mbar_drain(&b_wfull[i % a.nstage], (uint32_t)(i / a.nstage) & 1u)) atomicMax(a.err, 1);
     } else if (warp == kZbMmaWarp) {
         // ---- MMA issue ----
         if (lane == 0) {

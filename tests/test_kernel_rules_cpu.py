@@ -112,3 +112,14 @@ def test_read_out_warps_of_the_convolution_give_up_together(tmp_path):
     subprocess.run(["g++", "-std=c++20", "-O1", "-pthread", str(cpp), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
+
+
+def test_convolution_waits_for_every_bulk_copy():
+    """The thread that issues the weights' bulk copies waits for the last of
+    each buffer whatever became of the other roles (one of them may give up
+    after this thread is through), so no copy lands in shared memory that
+    another CTA already owns."""
+    body = kernels("unet.cu")["k_conv_zb"]
+    staging = body[:body.index("mbar_drain(&b_wfull")]
+    tail = staging[staging.rindex("cp_async_wait_all();"):]
+    assert "s_abort" not in tail and "if (pt == 0)" in tail
