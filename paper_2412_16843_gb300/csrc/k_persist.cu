@@ -26,6 +26,8 @@
 #include "ops.cuh"
 #include "../../include/cdi.h"
 
+#include <algorithm>
+
 namespace cdi {
 
 namespace {
@@ -835,6 +837,21 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_tail(const __grid_consta
     tail_vcycle<float, DIM>(A, true, reinterpret_cast<float*>(smd));
 }
 
+// Let fn be launched with smem bytes of dynamic shared memory.  The limit belongs to the function, for all contexts,
+// batches and threads of the process, so it is always set to the most a CTA may have (what a launch asks for is its
+// own); smem beyond that is refused.
+static cudaError_t allow_smem(const void* fn, size_t smem) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes at{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess) return e;
+    const size_t most = (size_t)optin - std::min((size_t)optin, at.sharedSizeBytes);
+    if (smem > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 static void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, int clusters, int threads,
                                   size_t smem, cudaStream_t s) {
     cfg.gridDim = dim3((unsigned)(cluster * clusters));
@@ -864,7 +881,7 @@ static int largest_cluster(const void* fn, int threads, size_t smem) {
 
 cudaError_t tail_prepare(int dim, size_t smem) {
     const void* fn = (dim == 2) ? (const void*)k_tail<2> : (const void*)k_tail<3>;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return allow_smem(fn, smem);
 }
 
 cudaError_t launch_tail(const InstArgs<float>& A, int dim, size_t smem, cudaStream_t s) {
@@ -890,7 +907,7 @@ cudaError_t launch_step_persist(PersistArgs<T>& A, size_t smem, int grid, int cl
 template <typename T>
 cudaError_t persist_prepare(int dim, size_t smem, int* grid, int* cluster) {
     const void* fn = (dim == 2) ? (const void*)k_step_persist<T, 2> : (const void*)k_step_persist<T, 3>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -900,7 +917,7 @@ cudaError_t persist_prepare(int dim, size_t smem, int* grid, int* cluster) {
     *grid = nsm;  // one CTA per SM
     fn = (dim == 2) ? (const void*)k_step_cluster<T, 2> : (const void*)k_step_cluster<T, 3>;
     *cluster = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
+    if (allow_smem(fn, smem) == cudaSuccess)
         *cluster = largest_cluster(fn, kPersistThreads, smem);
     else
         cudaGetLastError();
@@ -924,7 +941,7 @@ static const void* batch_fn_threads(int dim, int threads, bool cluster) {
 template <typename T>
 cudaError_t batch_prepare(int dim, int threads, size_t smem, int cluster, int* groups) {
     const void* fn = batch_fn_threads<T>(dim, threads, cluster > 1);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
