@@ -104,6 +104,7 @@ struct GridX {
     int red;
     unsigned long long epoch;  // barriers passed by this CTA
     using Ld = LG;
+    static constexpr bool kTailCall = false;
     // consecutive groups of 32 cells go to consecutive CTAs: a grid of fewer cells than threads is spread over all
     // SMs instead of filling the first few (their FP64 pipes bind the stage phases: the cell phase of a 64 x 32 grid
     // took 33k cycles on four SMs)
@@ -176,6 +177,7 @@ struct GridX {
 
 struct BlockX {
     using Ld = LP;  // one CTA owns the instance: its own writes are visible after __syncthreads
+    static constexpr bool kTailCall = true;
     __device__ int tid() const { return threadIdx.x; }
     __device__ int nth() const { return blockDim.x; }
     __device__ int spread() const { return threadIdx.x; }
@@ -198,6 +200,7 @@ struct ClusterX {
     double* slots;  // this CTA's shared memory, [2][kMaxCluster]: the cluster's partials
     int red;
     using Ld = LG;
+    static constexpr bool kTailCall = false;
     __device__ int tid() const { return (int)(((threadIdx.x >> 5) * size + rank) * 32 + (threadIdx.x & 31)); }
     __device__ int nth() const { return (int)(size * blockDim.x); }
     __device__ int spread() const { return (int)(threadIdx.x * size + rank); }
@@ -249,6 +252,11 @@ struct ClusterX {
         asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
         return r;
     }
+};
+
+// the cluster of a batched instance
+struct BatchClusterX : ClusterX {
+    static constexpr bool kTailCall = true;
 };
 
 // ---------------------------------------------------------------------------
@@ -399,6 +407,18 @@ __device__ void tail_vcycle(const InstArgs<T>& A, bool first, float* sm) {
     }
 }
 
+// The tail as a call, for the batched kernels: inlined, its coarse solve made
+// those of 64 registers a thread spill through the step's cell loops.
+// k_batch_persist<float, 2, 1024>: 438 / 840 bytes of spill stores / loads ->
+// 248 / 576; 512 instances 36.9 -> 34.4 ms a step (512 threads 55.7 -> 51.6;
+// 256 threads, which spill nothing but take 208 registers, 99.9 -> 91.5), 64 on
+// clusters of 8 7.9 -> 7.6.  The kernels of a single grid keep it inlined (as a
+// call 64 x 32 FP64 steps on its cluster in 0.89 instead of 0.83 ms).
+template <typename T, int DIM>
+__device__ __noinline__ void tail_vcycle_call(const InstArgs<T>& A, bool first, float* sm) {
+    tail_vcycle<T, DIM>(A, first, sm);
+}
+
 // One FP32 V-cycle on the correction equation A e = r from level 0 (levels
 // 0 .. lt-1 by the executor's threads, the tail by one CTA), ending with
 // p += e.  Every grid-wide level starts with its red cells already at their
@@ -439,7 +459,10 @@ __device__ bool vcycle(const InstArgs<T>& A, X& x, bool first, float* sm) {
         }
         if (!x.sync()) return false;
     }
-    if (x.tail_cta()) tail_vcycle<T, DIM>(A, first, sm);
+    if (x.tail_cta()) {
+        if constexpr (X::kTailCall) tail_vcycle_call<T, DIM>(A, first, sm);
+        else tail_vcycle<T, DIM>(A, first, sm);
+    }
     if (!x.sync()) return false;
     const MGLevel L0 = A.lv[0];
     PT<T>* P0 = ops::pbuf<T>(L0);
@@ -793,7 +816,7 @@ __global__ void __launch_bounds__(NT, 1) k_batch_cluster(BatchArgs<T> B) {
         int4* dst = reinterpret_cast<int4*>(&sA);
         for (int w = threadIdx.x; w < (int)(sizeof(InstArgs<T>) / sizeof(int4)); w += blockDim.x) dst[w] = src[w];
         __syncthreads();
-        ClusterX x{rank, size, s_slots, 0};
+        BatchClusterX x{{rank, size, s_slots, 0}};
         run_steps<T, DIM>(sA, x, B.nsteps, B.stats + i, sm);
     }
 }
