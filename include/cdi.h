@@ -292,7 +292,11 @@ void cdi_destroy(cdi_ctx* ctx);
  * one instance (largest first) and runs all its steps, so instances never
  * wait for each other.  The arithmetic of every instance is that of cdi_step
  * (Sec. 4 time step), so results equal those of stepping each context alone
- * up to the order of the sums over the grid.  All instances need the same dimension and precision and
+ * up to the order of the sums over the grid.  That order follows from the CTAs
+ * an instance runs on (cdi_batch_cluster), which one choice for the whole batch
+ * sets from all its instances' sizes, the threads per CTA, the tail budget and
+ * the device: an instance's last bits may change when others are added,
+ * removed or resized.  All instances need the same dimension and precision and
  * must stay alive while the batch exists.
  * ------------------------------------------------------------------------- */
 typedef struct cdi_batch cdi_batch;
@@ -334,6 +338,10 @@ cdi_status cdi_batch_autotune(cdi_batch* b, const double* dt, int trial_steps,
  * count of one solve, total V-cycles; and the launch's device time (ms). */
 cdi_status cdi_batch_stats(cdi_batch* b, int i, int* status, int* max_vcycles,
                            int* total_vcycles, float* last_ms);
+
+/* CTAs each instance ran on in the last cdi_batch_step (1, 2, 4, 8 or 16; 1
+ * before the first step). */
+cdi_status cdi_batch_cluster(const cdi_batch* b, int* ctas);
 
 /* Last error of the batch (NULL: of the last failed cdi_batch_create). */
 const char* cdi_batch_last_error(const cdi_batch* b);

@@ -96,6 +96,7 @@ def load(path: str = LIB_PATH):
         "cdi_batch_autotune": [P, DP, I, IP, ctypes.POINTER(S), DP],
         "cdi_batch_set_tail_budget": [P, S],
         "cdi_batch_stats": [P, I, IP, IP, IP, ctypes.POINTER(ctypes.c_float)],
+        "cdi_batch_cluster": [P, IP],
         "cdi_unet_create": [ctypes.POINTER(P), I, I, I],
         "cdi_unet_workspace_bytes": [P, ctypes.POINTER(S)],
         "cdi_unet_bind_workspace": [P, P, S, P],
@@ -396,6 +397,12 @@ class Batch:
         self._check(self.lib.cdi_batch_stats(self.h, i, ctypes.byref(st), ctypes.byref(mx), ctypes.byref(tot),
                                              ctypes.byref(ms)))
         return {"status": st.value, "max_cycles": mx.value, "total_cycles": tot.value, "last_ms": ms.value}
+
+    def cluster(self):
+        """CTAs each instance ran on in the last step."""
+        n = ctypes.c_int()
+        self._check(self.lib.cdi_batch_cluster(self.h, ctypes.byref(n)))
+        return n.value
 
 
 class Unet:

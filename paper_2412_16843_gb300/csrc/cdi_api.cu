@@ -9,6 +9,7 @@
 //       projection: f = div u*/(c dt), multigrid, u = u* - c dt grad p/rho_f
 // The new state lands in the stage buffers, whose role is then swapped with
 // the state buffers.
+#include "batch_split.cuh"
 #include "cdi_internal.cuh"
 #include "unet.cuh"
 #include "../../include/cdi.h"
@@ -20,7 +21,6 @@
 #include <string>
 #include <vector>
 #include <algorithm>
-#include <functional>
 
 using namespace cdi;
 
@@ -1506,40 +1506,22 @@ void batch_carve(cdi_batch* b, char* base, size_t* total) {
     *total = cv.off + 256;
 }
 
-// CTAs an instance, and how many instances run at once.  One CTA an instance does the most work a second when
-// instances abound, but the launch ends with its slowest instance: of 64 instances of 2k to 131k cells the largest
-// was alone on one SM for most of the launch.  Larger clusters shorten that tail and leave fewer slots.  The
-// instances (largest first) are laid out over the slots of every cluster size, a step of c cells on n CTAs taken as
-// 0.2 us (1 + 0.03 (n - 1)) c / n plus 0.4 ms of barriers and shared-memory multigrid tails (fitted to the FP32 sweep
-// at 1024 threads); the size with the earliest end is taken, a larger one only for a gain of 5 %.
-// Measured there (ms a step of the whole batch, clusters of 1 / 2 / 4 / 8 / 16; resident clusters on 152 SMs: 152 / 76 /
-// 36 / 15 / 7): 64 instances 25.9 / 15.1 / 8.5 / 9.0 / 15.5, 160 instances 31.8 / 18.4 / 13.7 / 23.1 / 40.0, 512 instances
-// 36.8 / 34.3 / 43.2 / 73.3 / 127.
+// CTAs an instance (batch_split.cuh), and how many instances run at once
 template <typename T>
 cudaError_t batch_split(cdi_batch* b) {
-    double best = 0.0;
-    for (int n = 1; n <= kMaxCluster; n *= 2) {
-        int groups = 0;
-        const cudaError_t e = batch_prepare<T>(b->dim, b->threads, b->smem, n, &groups);
-        if (e != cudaSuccess) {
-            if (n == 1) return e;
-            cudaGetLastError();  // this cluster size does not fit: keep the smaller one
-            break;
-        }
-        groups = std::min(groups, b->n);
-        std::vector<double> end(groups, 0.0);  // a min-heap of the slots' ends
-        for (int k = 0; k < b->n; ++k) {
-            std::pop_heap(end.begin(), end.end(), std::greater<double>());
-            end.back() += 0.2 * (1.0 + 0.03 * (n - 1)) * (double)b->inst[b->order[k]]->g.N / n + 400.0;
-            std::push_heap(end.begin(), end.end(), std::greater<double>());
-        }
-        const double t = *std::max_element(end.begin(), end.end());
-        if (n == 1 || t < 0.95 * best) {
-            best = t;
-            b->cluster = n;
-            b->groups = groups;
-        }
+    int slots[8], sizes = 0;
+    for (int n = 1; n <= kMaxCluster; n *= 2, ++sizes) {
+        const cudaError_t e = batch_prepare<T>(b->dim, b->threads, b->smem, n, &slots[sizes]);
+        if (e == cudaSuccess) continue;
+        if (n == 1) return e;
+        cudaGetLastError();  // this cluster size does not fit: a smaller one
+        break;
     }
+    std::vector<long> cells(b->n);
+    for (int k = 0; k < b->n; ++k) cells[k] = b->inst[b->order[k]]->g.N;
+    const int k = batch_split_choice(cells.data(), b->n, slots, sizes, sizeof(T) == 8, b->threads);
+    b->cluster = 1 << k;
+    b->groups = std::min(slots[k], b->n);
     return cudaSuccess;
 }
 
@@ -1765,6 +1747,12 @@ cdi_status cdi_batch_stats(cdi_batch* b, int i, int* status, int* max_vcycles, i
     if (max_vcycles) *max_vcycles = b->stats[i].max_cycles;
     if (total_vcycles) *total_vcycles = b->stats[i].total_cycles;
     if (last_ms) *last_ms = b->last_ms;
+    return CDI_OK;
+}
+
+cdi_status cdi_batch_cluster(const cdi_batch* b, int* ctas) {
+    if (!b || !ctas) return bfail(nullptr, CDI_EINVAL, "null argument");
+    *ctas = b->cluster;
     return CDI_OK;
 }
 
