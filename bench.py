@@ -614,7 +614,7 @@ def forms_report(steps=30):
     for w in wls:
         sv = cdi.from_workload(w, precision=cdi.FP32_MIXED, tol=PRESSURE_TOL)
         sv.set_solver(PRESSURE_TOL, 100, cdi.WARM_EXTRAP)
-        sv.set_smoothing(2, 2)  # one CTA per instance: barriers are cheap, fewer V-cycles win (measured)
+        sv.set_smoothing(2, 2)  # CTA or cluster barriers are cheap, fewer V-cycles win (measured)
         solvers.append(sv)
     b = cdi.Batch(solvers)
     dts = np.array([w.dt for w in wls])

@@ -10,18 +10,21 @@
 //   same convergence decision.  Data another CTA wrote before the last barrier
 //   is read with ld.global.cg (L2), never from a possibly stale L1 line.
 //
+// k_step_cluster: the same on one thread-block cluster of 8 or 16 CTAs, for the
+//   smallest grids (hardware cluster barriers, reductions through distributed
+//   shared memory).
+//
 // k_batch_persist: many independent grids (a parameter sweep) in one launch.
 //   Each CTA takes the largest instance not yet taken (atomic counter over a
 //   size-sorted descriptor array) and runs all its steps alone, so every
 //   barrier is a __syncthreads and no CTA ever waits for another.
 //
-// k_batch_cluster: the same with a thread-block cluster in the place of a CTA
-//   (barriers are hardware cluster barriers, reductions go through distributed
-//   shared memory), for batches whose largest instances would outlast the rest
-//   on one SM each.
+// k_batch_cluster: the same with a thread-block cluster of 2 to 16 CTAs in the
+//   place of a CTA, one size for the whole launch, for batches whose largest
+//   instances would outlast the rest on one SM each (batch_split.cuh).
 //
 // All run the same step code, written once against an executor X that
-// supplies the thread range, the barrier and the reductions.  In both, the
+// supplies the thread range, the barrier and the reductions.  In all, the
 // multigrid levels that fit in shared memory are solved by one CTA there.
 #include "ops.cuh"
 #include "../../include/cdi.h"

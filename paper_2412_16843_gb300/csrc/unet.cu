@@ -1,17 +1,22 @@
 // Warm-start U-Net on the tensor cores: forward, backward and Adam.
 //
 // Convolutions are implicit GEMMs on channels-last BF16 activations
-// [voxel][channel] with mma.sync m16n8k16 (BF16 in, FP32 accumulate):
+// [voxel][channel] with FP32 accumulation:
 //   forward      y[v][co] = b[co] + sum_t sum_ci x[v + off(t)][ci] W[t][co][ci]
-//                (M = 16 voxels per warp, N = all output channels, K = 27 taps x Cin)
 //   data grad    dx = forward(dy) with the taps flipped and W transposed,
 //                because the adjoint of a zero-padded correlation is the
 //                correlation with the mirrored kernel
 //   weight grad  dW[t][co][ci] = sum_v dy[v][co] x[v + off(t)][ci]
-//                (M = 16 output channels, N = input channels, K = voxels;
-//                partial sums of voxel chunks are added with atomics)
+// By default on tcgen05 with accumulators in tensor memory: k_conv_zb (forward
+// and data gradient; M = 128 voxels, the three dz taps folded into N) and
+// k_wgrad_tc (weight and bias gradients; M = rows of taps x input channels,
+// K = voxels, split sums added in a fixed order).  The alternative (k_conv,
+// k_wgrad) runs mma.sync m16n8k16: M = 16 voxels per warp, N = all output
+// channels, K = 27 taps x Cin, and for the weight gradient M = 16 output
+// channels, K = voxels, partial sums added with atomics.
 // Pooling (2x2x2 mean), nearest upsampling, channel concatenation, ReLU
-// masks, the mean-squared-error loss and Adam are elementwise kernels.
+// masks, the mean-squared-error loss and Adam are elementwise kernels; at
+// inference the last layer's read-out applies the 1x1x1 head.
 // Master weights and Adam moments are FP32; the tensor cores see BF16 copies.
 #include "unet.cuh"
 #include "ops.cuh"

@@ -4,6 +4,8 @@
     python -m paper_2412_16843_gb300.profile_cases unet 128     # network forward passes at 128^3
     python -m paper_2412_16843_gb300.profile_cases train 64     # 3 network training steps at 64^3
     python -m paper_2412_16843_gb300.profile_cases batch 64     # 64-instance FP32-mixed sweep, 3 steps
+    python -m paper_2412_16843_gb300.profile_cases couette 512  # 512x128 Couette, FP64, persistent, 3 steps
+    python -m paper_2412_16843_gb300.profile_cases small 64     # 64x32 drop, FP64, one cluster, 3 steps
     python -m paper_2412_16843_gb300.profile_cases drop3d 256   # 3D drop, FP32-mixed, separate kernels, 2 steps
     python -m paper_2412_16843_gb300.profile_cases wide 512 1   # 512x256x256 drop, FP32-mixed, previous-pressure
                                                                 # first guess, separate kernels, 1 step
@@ -55,6 +57,16 @@ def main(argv):
             b.step(dts, 1)
         torch.cuda.synchronize()
         print('batch ok', b.stats(0))
+    elif mode in ('couette', 'small'):
+        n = int(argv[2]) if len(argv) > 2 else (512 if mode == 'couette' else 64)
+        wl = inputs.couette_2d(n, n // 4, 1.0) if mode == 'couette' else inputs.drop_2d(n, n // 2)
+        s = cdi.from_workload(wl, tol=1e-8)
+        s.set_exec(cdi.EXEC_PERSISTENT)
+        s.set_solver(1e-8, 100, cdi.WARM_EXTRAP)
+        for _ in range(3):
+            s.step(wl.dt, 1)
+        torch.cuda.synchronize()
+        print(mode, 'ok', s.last_stats())
     elif mode == 'drop3d':
         n = int(argv[2]) if len(argv) > 2 else 256
         wl = inputs.drop_3d(n)
