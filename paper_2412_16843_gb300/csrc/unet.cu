@@ -1004,7 +1004,9 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t mbar[2];
     __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
+    // a wait gave up: in an even chunk, an odd chunk, after the chunks.  One word for all would let a fast thread set it
+    // in its next wait before a slow one has read it after this chunk's barrier, and the two wait at other barriers.
+    __shared__ int s_abort[3];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rb = blockIdx.x, nrb = gridDim.x;
     const int bstep = wg_bstep(N), bufb = wg_buf_bytes(N);
@@ -1018,7 +1020,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
     if (tid == 0) {
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);
-        s_abort = 0;
+        s_abort[0] = s_abort[1] = s_abort[2] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
@@ -1034,10 +1036,10 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
     bool pending[2] = {false, false};
     bool unconfirmed[2] = {false, false};
     uint32_t uphase[2] = {0u, 0u};
-    auto wait_mma = [&](int b) {
+    auto wait_mma = [&](int b, int flag) {
         if (pending[b]) {
             if (!mbar_wait_bounded(&mbar[b], phase[b])) {
-                s_abort = 1;
+                s_abort[flag] = 1;
                 atomicExch(err, 1);
                 unconfirmed[b] = true;
                 uphase[b] = phase[b];
@@ -1116,11 +1118,11 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
 
     for (int c = 0; c < nch; ++c) {
         const int b = c & 1;
-        wait_mma(b);  // the MMAs of chunk c - 2 read this buffer
+        wait_mma(b, b);  // the MMAs of chunk c - 2 read this buffer
         stage(c, b);
         fence_proxy_async();
         __syncthreads();
-        if (s_abort) break;
+        if (s_abort[b]) break;
         if (tid == 0) {
             tc_fence_after();
             const uint32_t a0 = smem_u32(smem + b * bufb), b0 = a0 + kWgABytes;
@@ -1134,9 +1136,9 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(CG g, const bf16* __res
         }
         pending[b] = true;
     }
-    for (int b = 0; b < 2; ++b) wait_mma(b);
+    for (int b = 0; b < 2; ++b) wait_mma(b, 2);
     __syncthreads();
-    if (!s_abort && nch > 0 && warp < 4) {
+    if (!(s_abort[0] | s_abort[1] | s_abort[2]) && nch > 0 && warp < 4) {
         tc_fence_after();
         const int row = warp * 32 + lane;
         float* dst = part + ((size_t)(blockIdx.y * nrb + rb) * 128 + row) * N;

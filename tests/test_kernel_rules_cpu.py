@@ -123,3 +123,16 @@ def test_convolution_waits_for_every_bulk_copy():
     staging = body[:body.index("mbar_drain(&b_wfull")]
     tail = staging[staging.rindex("cp_async_wait_all();"):]
     assert "s_abort" not in tail and "if (pt == 0)" in tail
+
+
+def test_weight_gradient_ctas_give_up_together():
+    """After a chunk's barrier every thread of a CTA reads whether a wait gave up;
+    a fast thread may by then be in its next wait.  So consecutive chunks, and
+    the waits after the last, write other words than the one being read:
+    threads that disagree would wait at different barriers."""
+    body = kernels("unet.cu")["k_wgrad_tc"]
+    assert re.search(r"__shared__ int s_abort\[3\]", body) and "s_abort[flag] = 1" in body
+    loop = body[body.index("for (int c = 0; c < nch; ++c)"):]
+    assert re.search(r"const int b = c & 1;\s+wait_mma\(b, b\);", loop)
+    assert re.search(r"__syncthreads\(\);\s+if \(s_abort\[b\]\) break;", loop)
+    assert re.search(r"wait_mma\(b, 2\);\s+__syncthreads\(\);", loop)
